@@ -73,6 +73,13 @@ void ho_loss_terms(int n, const std::vector<Row> &Ho, long long *C4, long long *
 
 int gf2_rank(std::vector<Row> rows, int n);
 
+// Row/column kernels (rc_device.cuh): the lengths of the code's index tables.
+constexpr int kRcConstBytes = 60000;  // constant-memory tables of the 32-slot kernel
+struct RcTables {
+  int const_bytes = 0, rows16 = 0, cols16 = 0, kw = 0;
+};
+int rc_threads(int slots, int tasks);
+
 uint64_t splitmix64_next(uint64_t *state);
 uint64_t splitmix64_mix(uint64_t z);
 void draw_autos_host(int n, int P, uint64_t seed, uint64_t frame0, int F, uint16_t *out);
@@ -96,9 +103,12 @@ struct bch_code {
   };
   mutable std::vector<JitMemo> jit_memo;
   mutable std::mutex jit_mu;
+  bchlib::RcTables rc;  // row/column kernels' table lengths
 };
 
 namespace bchlib {
+RcTables rc_tables(const bch_code *c);
+
 void set_error(const std::string &msg);
 bch_status fail(bch_status s, const std::string &msg);
 // Counts one kernel launch of the library (bch_kernel_launches reports the total).

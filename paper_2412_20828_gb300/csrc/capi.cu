@@ -13,11 +13,13 @@
 #include <vector>
 
 #include "bch_kernels.cuh"
+#include "rc_layout.h"
 
 using namespace bchlib;
 
 namespace bchlib {
 cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac = 0);
+cudaKernel_t jit_rc_kernel(const bch_code *c, int msg, int qfrac, int FB, int P, std::string *err);
 bool jit_compile_check(const bch_code *c, int msg, std::string *log);
 bool jit_serve_compile_check(const bch_code *const *codes, int n_codes, std::string *log);
 int jit_block_size(int n);
@@ -310,6 +312,7 @@ bch_status upload_code(bch_code *c) {
   c->dev_blob = blob;
   c->dc = dc;
   c->dev_dc = reinterpret_cast<DevCode *>(b + off_desc);
+  c->rc = rc_tables(c);
   return BCH_OK;
 }
 
@@ -701,9 +704,74 @@ static cudaError_t launch_jit(cudaKernel_t k, const bch_code *code, const NmsArg
   return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
 }
 
+// ---- row/column kernels (rc_device.cuh)
+static size_t rc_smem_bytes(const bch_code *code, const NmsArgs &a, int FB) {
+  return size_t(rc_layout(code->alg.n, a.P, int(code->rows.size()), FB, a.msg == BCH_MSG_INT8 ? 3 : 2,
+                          code->rc.kw, code->rc.rows16, code->rc.cols16).words) * 4;
+}
+
+static bool rc_fits(const bch_code *code, const NmsArgs &a, int FB) {
+  return rc_smem_bytes(code, a, FB) <= 227 * 1024 && (FB < 32 || code->rc.const_bytes <= kRcConstBytes);
+}
+
+// The row/column kernel (frame slots per block: 1 or 32) for this call, or 0 when the
+// one-thread-per-frame kernel is the better one.  BCHDEC_JIT_RC=0|1|32 overrides (a tuning
+// and comparison knob; all compute the same bits).  The lines lie where the measured times
+// cross (GB300, 12 iterations, Eb/N0 U[1, 6) dB unless said; us for 1 slot / 32 slots / one
+// thread per frame; ep = edges x copies of one iteration):
+//  * one slot up to 8 + 61200 / ep frames per SM: BCH(63,36), ep 2550, 4096 frames 77 / 91 /
+//    349, 16 384 frames 300+ / 182 / 350; BCH(127,64), ep 8670, 1531 frames 138 / 218 / 1322,
+//    4096 frames 310 / 219 / 1322; BCH(63,36) with 9 copies 2400 frames 90 / 109 / 321, 4800
+//    frames 163 / 110 / 322;
+//  * n <= 63, three copies: 32 slots up to 160 (FP16 300, INT8 176) frames per SM, the crossing
+//    where every frame is hard (1 to 2 dB: 20 000 frames - / 306 / 351, 30 000 - / 424 / 354);
+//    other numbers of copies, whose loops are not unrolled, up to 64;
+//  * beyond ~1000 edges the straight-line rows outgrow the instruction cache and 32 slots win
+//    at any size: BCH(127,64) 100 000 frames - / 2731 / 5384, BCH(127,99) - / 2156 / 4232,
+//    BCH(63,36) with 122 rows 200 000 frames - / 2032 / 2827;
+//  * where the copies of 32 frames exceed shared memory (n = 127, five copies or more) one
+//    slot wins up to about 112 frames per SM: nine copies 10 000 frames 822 / - / 1318, 25 000
+//    frames 2011 / - / 2000.
+static int rc_slots(const bch_code *code, const NmsArgs &a, int sms) {
+  if (const char *v = std::getenv("BCHDEC_JIT_RC")) {
+    const int fb = std::atoi(v);
+    return (fb == 1 || fb == 32) && rc_fits(code, a, fb) ? fb : 0;
+  }
+  const bool fits32 = rc_fits(code, a, 32), cached = code->alg.n <= 63 && code->dc.edges <= 1000;
+  const int ep = std::max(1, code->dc.edges * a.P), one = fits32 || cached ? std::min(64, 8 + 61200 / ep) : 112;
+  if (a.F <= sms * one && rc_fits(code, a, 1)) return 1;
+  if (!fits32) return 0;
+  const int many = a.P != 3 ? 64 : a.msg == BCH_MSG_FP16 ? 300 : a.msg == BCH_MSG_INT8 ? 176 : 160;
+  return !cached || a.F <= sms * many ? 32 : 0;
+}
+
+static cudaError_t launch_rc(cudaKernel_t k, int FB, const bch_code *code, const NmsArgs &a, cudaStream_t st) {
+  const void *fn = reinterpret_cast<const void *>(k);
+  const size_t smem = rc_smem_bytes(code, a, FB);
+  const int tpb = rc_threads(FB, a.P * std::max(code->alg.n, int(code->rows.size())));
+  int sms = 0, per_sm = 0;
+  cudaError_t e = launch_geometry(fn, tpb, smem, &sms, &per_sm);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const long long need = (a.F + FB - 1) / FB, blocks = std::min<long long>(need, (long long)sms * per_sm);
+  void *args[] = {const_cast<NmsArgs *>(&a)};
+  note_launch();
+  return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
+}
+
 static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaStream_t st,
                                    std::string *why) {
   const int mode = kernel_mode();
+  if (a.P > 0 && mode != 1) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int fb = rc_slots(code, a, sms);
+    std::string err;
+    if (fb)
+      if (cudaKernel_t k = jit_rc_kernel(code, a.msg, a.qfrac, fb, a.P, &err)) return launch_rc(k, fb, code, a, st);
+  }
   // auto and jit: the specialised kernel (for n = 127 it spills but still runs 1.8x
   // faster than the precompiled one; its first compile takes tens of seconds and is
   // cached on disk); auto falls back to the precompiled kernel if it does not compile

@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include "bch_internal.h"
+#include "rc_layout.h"
 
 namespace bchlib {
 
@@ -39,6 +40,8 @@ extern const char kNmsDeviceText[];
 extern const char kAutosDeviceText[];
 extern const char kOsdDeviceText[];
 extern const char kServeDeviceText[];
+extern const char kRcLayoutText[];
+extern const char kRcDeviceText[];
 
 namespace {
 
@@ -619,6 +622,130 @@ static std::string jit_body_source(const bch_code *c, int msg) {
   return o.str();
 }
 
+
+// ---- row/column kernels (rc_device.cuh) with one or 32 frame slots per block.
+// 512 threads with 32 slots: 640, 768 and 1024 measured 1-4% slower at 4096 .. 100 000
+// frames of BCH(63,36), (127,64) and (127,99) (more warps do not shorten the shared-memory
+// and ALU time that bounds the passes).  With one slot about one task per thread (P
+// max(rows, n) tasks).
+int rc_threads(int FB, int tasks) { return FB == 32 ? 512 : std::min(512, std::max(64, (tasks + 31) & ~31)); }
+
+// The graph's tables: rows grouped by weight (stable), states numbered in that order;
+// columns in order of their degree padded to a multiple of 4, each listing its row states
+// in the code's row order (the order of the additions).  For 32 slots the entries are byte
+// offsets scaled for the [index][slot] arrays, four to a constant-memory word; else 16-bit
+// indices, four to a word, laid out so that lanes on consecutive rows or columns read
+// consecutive words.
+static RcTables emit_rc_tables(std::ostringstream &o, const bch_code *c, int FB, std::string *calls) {
+  const int n = c->alg.n, M = int(c->rows.size()), K = int(c->alg.std_h.size());
+  std::vector<int> order(M), state(M), corder(n);
+  for (int i = 0; i < M; i++) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return c->rows[a].weight() < c->rows[b].weight(); });
+  std::vector<std::vector<int>> by_row(M), by_col(n);
+  for (int i = 0; i < M; i++) {
+    state[order[i]] = i;
+    for (int u = 0; u < n; u++)
+      if (c->rows[order[i]].get(u)) by_row[i].push_back(u);
+  }
+  size_t w4 = 0, d4 = 0;
+  for (const auto &r : by_row) w4 = std::max(w4, (r.size() + 3) / 4);
+  for (int u = 0; u < n; u++) {
+    corder[u] = u;
+    for (int r = 0; r < M; r++)
+      if (c->rows[r].get(u)) by_col[u].push_back(state[r]);
+    while (by_col[u].empty() || by_col[u].size() % 4) by_col[u].push_back(M);  // the neutral row
+    d4 = std::max(d4, by_col[u].size() / 4);
+  }
+  std::stable_sort(corder.begin(), corder.end(), [&](int a, int b) { return by_col[a].size() < by_col[b].size(); });
+  RcTables info;
+  info.kw = (K + 31) / 32;
+  info.rows16 = int(w4 * M * 4);
+  info.cols16 = int(4 * size_t((n + 1) / 2) + d4 * n * 4);
+  std::ostringstream rows, cols, rcalls, ccalls;
+  size_t rt = 0, ct = 0;
+  for (int i = 0; i < M;) {
+    const size_t w = by_row[i].size();
+    int e = i;
+    while (e < M && by_row[e].size() == w) e++;
+    rcalls << "  rc_rows<MSG, " << w << ">(c, " << e - i << ", " << i << ", " << rt << ");\n";
+    for (int r = i; r < e; r++)
+      for (size_t q = 0; q < ((w + 3) & ~size_t(3)); q++)
+        if (FB == 32) rows << (q % 4 ? "" : "{") << (q < w ? by_row[r][q] * 128 : 0) << (q % 4 == 3 ? "}," : ",");
+    rt += size_t(e - i) * ((w + 3) / 4);
+    i = e;
+  }
+  for (int i = 0; i < n;) {
+    const size_t d = by_col[corder[i]].size();
+    int e = i;
+    while (e < n && by_col[corder[e]].size() == d) e++;
+    ccalls << "  rc_cols<MSG, " << d / 4 << ">(c, " << e - i << ", " << i << ", " << ct << ");\n";
+    for (int k = i; k < e; k++)
+      if (FB == 32) {
+        cols << "{" << corder[k] * 128 << ",0,0,0},";
+        for (size_t q = 0; q < d; q++)
+          cols << (q % 4 ? "" : "{") << by_col[corder[k]][q] * 32 << (q % 4 == 3 ? "}," : ",");
+      }
+    ct += size_t(e - i) * (d / 4 + 1);
+    i = e;
+  }
+  info.const_bytes = int((rt + ct) * 16);
+  if (FB < 32) {
+    for (size_t q = 0; q < w4; q++)
+      for (int r = 0; r < M; r++)
+        for (size_t h = 4 * q; h < 4 * q + 4; h++) rows << (h < by_row[r].size() ? by_row[r][h] : n) << ",";
+    for (int i = 0; i < 2 * ((n + 1) / 2); i++)
+      cols << (i < n ? corder[i] : 0) << "," << (i < n ? by_col[corder[i]].size() / 4 : 0) << ",";
+    for (size_t q = 0; q < d4; q++)
+      for (int i = 0; i < n; i++)
+        for (size_t h = 4 * q; h < 4 * q + 4; h++) {
+          const auto &v = by_col[corder[i]];
+          cols << (h < v.size() ? v[h] : M) << ",";
+        }
+  }
+  o << "#define RC_N " << n << "\n#define RC_M " << c->alg.m << "\n#define RC_R " << M << "\n#define RC_KW " << info.kw
+    << "\n#define RC_W4 " << w4 << "\n#define RC_ROWTAB16 " << info.rows16 << "\n#define RC_COLTAB16 " << info.cols16
+    << "\n__device__ const uint32_t rc_cmask[] = {";
+  for (int u = 0; u < n; u++)
+    for (int w = 0; w < info.kw; w++) {
+      uint32_t v = 0;
+      for (int r = 32 * w; r < std::min(K, 32 * w + 32); r++) v |= uint32_t(c->alg.std_h[r].get(u)) << (r - 32 * w);
+      o << v << "u,";
+    }
+  if (FB == 32)
+    o << "};\n__constant__ int4 rc_rowtab[] = {" << rows.str() << "};\n__constant__ int4 rc_coltab[] = {" << cols.str()
+      << "};\n";
+  else
+    o << "};\n__device__ __align__(16) const unsigned short rc_rowtab16[] = {" << rows.str()
+      << "};\n__device__ __align__(16) const unsigned short rc_coltab16[] = {" << cols.str() << "};\n";
+  if (FB == 32)
+    *calls = "template <int MSG>\n__device__ __forceinline__ void rc_row_pass(const RcPtr &c) {\n" + rcalls.str() +
+             "}\ntemplate <int MSG>\n__device__ __forceinline__ void rc_column_pass(const RcPtr &c) {\n" + ccalls.str() +
+             "}\n";
+  return info;
+}
+
+RcTables rc_tables(const bch_code *c) {
+  std::ostringstream o;
+  std::string calls;
+  return emit_rc_tables(o, c, 32, &calls);
+}
+
+// The source of one row/column kernel: FB slots, PC copies (0: any number).
+static std::string jit_rc_source(const bch_code *c, int msg, int qfrac, int FB, int PC) {
+  std::ostringstream o, tab;
+  std::string calls;
+  emit_rc_tables(tab, c, FB, &calls);
+  o << "#define BCH_JIT_QFRAC " << qfrac << "\n#define RC_FB " << FB << "\n#define RC_PC " << PC << "\n";
+  emit_prologue(o, msg, false);
+  o << "}  // namespace bchlib\n" << tab.str() << kRcLayoutText << "\n" << kRcDeviceText << "\nnamespace bchlib {\n"
+    << calls << "}  // namespace bchlib\n"
+    << "extern \"C\" __global__ void __launch_bounds__(" << 512 << ", "
+    << (FB == 32 && c->alg.n <= 63 ? 2 : 1) << ") bch_nms_rc(const bchlib::NmsArgs a) {\n"
+    << "  extern __shared__ __align__(16) unsigned char smem[];\n  bchlib::rc_persistent<" << msg
+    << ">(a, reinterpret_cast<uint32_t *>(smem));\n}\n";
+  return o.str();
+}
+
 // The serving kernel specialised to a server's codes (FP32 messages): one copy functor
 // per code on columns of stride 32 (one warp per block), row sums in registers for
 // n <= 63 and in the lane's scratch column for n = 127, dispatched on the warp's code.
@@ -836,6 +963,31 @@ cudaKernel_t jit_kernel_from_source(const bch_code *c, int msg, std::string *err
   return compile_source(jit_source(c, msg, qfrac), "bch_nms_jit", err);
 }
 
+// The row/column kernel of code c with FB slots per block for P copies;
+// nullptr with *err when it does not compile.  Three copies, the usual number, get a kernel
+// of their own (the copies' loops unrolled); any other number shares one.
+cudaKernel_t jit_rc_kernel(const bch_code *c, int msg, int qfrac, int FB, int P, std::string *err) {
+  const int PC = P == 3 ? 3 : 0;
+  const std::string key = "rc/" + std::to_string(msg) + "/" + std::to_string(qfrac) + "/" + std::to_string(FB) +
+                          "/" + std::to_string(PC);
+  {
+    std::lock_guard<std::mutex> lk(c->jit_mu);
+    for (const auto &m : c->jit_memo)
+      if (m.key == key) {
+        if (!m.kernel) *err = m.err;
+        return static_cast<cudaKernel_t>(m.kernel);
+      }
+  }
+  std::string why;
+  cudaKernel_t k = compile_source(jit_rc_source(c, msg, qfrac, FB, PC), "bch_nms_rc", &why);
+  {
+    std::lock_guard<std::mutex> lk(c->jit_mu);
+    c->jit_memo.push_back({key, static_cast<void *>(k), why});
+  }
+  if (!k) *err = why;
+  return k;
+}
+
 cudaKernel_t jit_serve_kernel(const bch_code *const *codes, int n_codes, std::string *err) {
   return compile_source(jit_serve_source(codes, n_codes), "bch_serve_jit", err);
 }
@@ -849,7 +1001,18 @@ cudaKernel_t jit_serve_blocks_kernel(const bch_code *const *codes, int n_codes, 
 static bool compile_check_source(const std::string &src, const char *entry, std::string *log);
 
 bool jit_compile_check(const bch_code *c, int msg, std::string *log) {
-  return compile_check_source(jit_source(c, msg, 0), "bch_nms_jit", log);
+  std::string rc_log;
+  for (int fb : {1, 32}) {  // the row/column kernels too
+    std::string one;
+    if (!compile_check_source(jit_rc_source(c, msg, 0, fb, 3), "bch_nms_rc", &one)) {
+      *log = one;
+      return false;
+    }
+    rc_log += one;
+  }
+  const bool ok = compile_check_source(jit_source(c, msg, 0), "bch_nms_jit", log);
+  *log += rc_log;
+  return ok;
 }
 
 bool jit_serve_compile_check(const bch_code *const *codes, int n_codes, std::string *log) {
@@ -865,9 +1028,11 @@ static bool compile_check_source(const std::string &src_in, const char *entry, s
     *log = api.err;
     return false;
   }
-  // BCHDEC_JIT_DUMP=<file>: also write the generated source there (a debugging aid)
+  // BCHDEC_JIT_DUMP=<file>: also write the generated source there (a debugging aid; the
+  // row/column kernels appended to <file>.rc)
   if (const char *dump = std::getenv("BCHDEC_JIT_DUMP")) {
-    if (FILE *fp = std::fopen(dump, "w")) {
+    const bool rc = std::strcmp(entry, "bch_nms_rc") == 0;
+    if (FILE *fp = std::fopen((std::string(dump) + (rc ? ".rc" : "")).c_str(), rc ? "a" : "w")) {
       std::fwrite(src.data(), 1, src.size(), fp);
       std::fclose(fp);
     }
