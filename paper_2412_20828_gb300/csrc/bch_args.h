@@ -34,19 +34,6 @@ struct GenArgs {
   uint64_t *codeword;
 };
 
-struct BwdArgs {
-  DevCode dc;
-  const uint16_t *autos;
-  int P;
-  const float *ckpt;
-  int ld, F, I;
-  const float *grad_out;
-  float *grad_llr;
-  float *partial;  // [blocks][I]
-  unsigned *check;  // checked builds: the device's check word [4]; else unused
-  float alpha[32];
-};
-
 // Parallel annealing chains of the H_o search (one block per chain).
 struct AnnealArgs {
   int n, Mo, steps, chains;
@@ -80,6 +67,8 @@ cudaError_t launch_bce(int n, const float *y, int ld, const uint64_t *cw, int F,
                        float *grad, float *partial, cudaStream_t st);
 size_t bce_workspace(int F);
 cudaError_t launch_backward(const BwdArgs &a, float *grad_alpha, cudaStream_t st);
+// grad_alpha[t] = sum of partial[0 .. nb)[t], in a fixed order.
+cudaError_t launch_reduce_alpha(const float *partial, int nb, int I, float *grad_alpha, cudaStream_t st);
 size_t backward_workspace(int F, int I);
 
 }  // namespace bchlib

@@ -50,4 +50,18 @@ struct NmsArgs {
   float alpha[32];  // alpha_t 2^qfrac
 };
 
+// Argument block of the backward kernels.
+struct BwdArgs {
+  DevCode dc;
+  const uint16_t *autos;
+  int P;
+  const float *ckpt;
+  int ld, F, I;
+  const float *grad_out;
+  float *grad_llr;
+  float *partial;  // [blocks][I]
+  unsigned *check;  // checked builds: the device's check word [4]; else unused
+  float alpha[32];
+};
+
 }  // namespace bchlib

@@ -20,6 +20,7 @@ using namespace bchlib;
 namespace bchlib {
 cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac = 0);
 cudaKernel_t jit_rc_kernel(const bch_code *c, int msg, int qfrac, int FB, int P, std::string *err);
+cudaKernel_t jit_rcb_kernel(const bch_code *c, std::string *err);
 bool jit_compile_check(const bch_code *c, int msg, std::string *log);
 bool jit_serve_compile_check(const bch_code *const *codes, int n_codes, std::string *log);
 int jit_block_size(int n);
@@ -785,6 +786,33 @@ static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaS
   return launch_nms(a, st);
 }
 
+// The backward pass: row by row on 32 frames per block (rc_backward.cuh), else (no run-time
+// compiler, BCHDEC_NMS_KERNEL=generic, or a matrix whose tables or row states do not fit) the
+// precompiled one-thread-per-frame kernel.  us, P = 3, 12 iterations, new / precompiled:
+// BCH(127,64) 256 frames 304 / 11 234, 65 536 frames 4 138 / 45 017; BCH(63,36) 256 frames 122 /
+// 3 314, 65 536 frames 1 680 / 7 585: no size prefers the precompiled one.
+static cudaError_t launch_backward_code(const bch_code *code, const BwdArgs &a, float *grad_alpha, cudaStream_t st) {
+  const int n = code->alg.n, R = int(code->rows.size());
+  const size_t smem = size_t(rcb_words(n, a.P, R, code->rc.w4, kRcbWarps, kRcbAcc)) * 4;
+  if (a.F > 0 && kernel_mode() != 1 && smem <= 227 * 1024 && code->rc.const_bytes <= kRcConstBytes) {
+    std::string err;
+    cudaKernel_t k = jit_rcb_kernel(code, &err);
+    if (k) {
+      const void *fn = reinterpret_cast<const void *>(k);
+      int sms = 0, per_sm = 0;
+      cudaError_t e = launch_geometry(fn, 32 * kRcbWarps, smem, &sms, &per_sm);
+      if (e != cudaSuccess) return e;
+      if (per_sm < 1) return cudaErrorInvalidConfiguration;
+      const int nb = std::min((a.F + 31) / 32, sms * per_sm);
+      void *args[] = {const_cast<BwdArgs *>(&a)};
+      note_launch();
+      e = cudaLaunchKernel(fn, dim3(unsigned(nb)), dim3(32 * kRcbWarps), args, smem, st);
+      return e == cudaSuccess ? launch_reduce_alpha(a.partial, nb, a.I, grad_alpha, st) : e;
+    }
+  }
+  return launch_backward(a, grad_alpha, st);
+}
+
 static bch_status run_nms(const bch_code *code, const bch_nms_params *params, const float *llr, int ld,
                           int n_frames, const uint16_t *autos, uint64_t *hard, uint8_t *iters,
                           uint8_t *flags, float *llr_out, float *ckpt, void *workspace,
@@ -945,7 +973,7 @@ bch_status bch_nms_backward(const bch_code *code, const bch_nms_params *params, 
   a.partial = reinterpret_cast<float *>(static_cast<unsigned char *>(workspace) + L.red);
   a.check = check_word();
   for (int t = 0; t < 32; t++) a.alpha[t] = t < params->iters ? params->alpha[t] : 0.0f;
-  BCH_CUDA(launch_backward(a, grad_alpha, static_cast<cudaStream_t>(stream)), "backward");
+  BCH_CUDA(launch_backward_code(code, a, grad_alpha, static_cast<cudaStream_t>(stream)), "backward");
   return BCH_OK;
 }
 

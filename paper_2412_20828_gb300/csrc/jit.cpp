@@ -42,6 +42,7 @@ extern const char kOsdDeviceText[];
 extern const char kServeDeviceText[];
 extern const char kRcLayoutText[];
 extern const char kRcDeviceText[];
+extern const char kRcBackwardText[];
 
 namespace {
 
@@ -636,7 +637,8 @@ int rc_threads(int FB, int tasks) { return FB == 32 ? 512 : std::min(512, std::m
 // offsets scaled for the [index][slot] arrays, four to a constant-memory word; else 16-bit
 // indices, four to a word, laid out so that lanes on consecutive rows or columns read
 // consecutive words.
-static RcTables emit_rc_tables(std::ostringstream &o, const bch_code *c, int FB, std::string *calls) {
+static RcTables emit_rc_tables(std::ostringstream &o, const bch_code *c, int FB, std::string *calls,
+                               std::string *bwd_calls = nullptr) {
   const int n = c->alg.n, M = int(c->rows.size()), K = int(c->alg.std_h.size());
   std::vector<int> order(M), state(M), corder(n);
   for (int i = 0; i < M; i++) order[i] = i;
@@ -659,15 +661,17 @@ static RcTables emit_rc_tables(std::ostringstream &o, const bch_code *c, int FB,
   std::stable_sort(corder.begin(), corder.end(), [&](int a, int b) { return by_col[a].size() < by_col[b].size(); });
   RcTables info;
   info.kw = (K + 31) / 32;
+  info.w4 = int(w4);
   info.rows16 = int(w4 * M * 4);
   info.cols16 = int(4 * size_t((n + 1) / 2) + d4 * n * 4);
-  std::ostringstream rows, cols, rcalls, ccalls;
+  std::ostringstream rows, cols, rcalls, ccalls, bcalls;
   size_t rt = 0, ct = 0;
   for (int i = 0; i < M;) {
     const size_t w = by_row[i].size();
     int e = i;
     while (e < M && by_row[e].size() == w) e++;
     rcalls << "  rc_rows<MSG, " << w << ">(c, " << e - i << ", " << i << ", " << rt << ");\n";
+    bcalls << "  rcb_rows<" << w << ">(c, " << e - i << ", " << i << ", " << rt << ");\n";
     for (int r = i; r < e; r++)
       for (size_t q = 0; q < ((w + 3) & ~size_t(3)); q++)
         if (FB == 32) rows << (q % 4 ? "" : "{") << (q < w ? by_row[r][q] * 128 : 0) << (q % 4 == 3 ? "}," : ",");
@@ -717,6 +721,14 @@ static RcTables emit_rc_tables(std::ostringstream &o, const bch_code *c, int FB,
   else
     o << "};\n__device__ __align__(16) const unsigned short rc_rowtab16[] = {" << rows.str()
       << "};\n__device__ __align__(16) const unsigned short rc_coltab16[] = {" << cols.str() << "};\n";
+  if (bwd_calls) {
+    o << "__device__ __align__(16) const unsigned short rcb_cols[] = {";
+    for (const auto &r : by_row)
+      for (size_t q = 0; q < 4 * w4; q++) o << (q < r.size() ? r[q] : 0) << ",";
+    o << "};\n";
+  }
+  if (bwd_calls)
+    *bwd_calls = "__device__ __forceinline__ void rcb_row_pass(RcbPtr &c) {\n" + bcalls.str() + "}\n";
   if (FB == 32)
     *calls = "template <int MSG>\n__device__ __forceinline__ void rc_row_pass(const RcPtr &c) {\n" + rcalls.str() +
              "}\ntemplate <int MSG>\n__device__ __forceinline__ void rc_column_pass(const RcPtr &c) {\n" + ccalls.str() +
@@ -743,6 +755,22 @@ static std::string jit_rc_source(const bch_code *c, int msg, int qfrac, int FB, 
     << (FB == 32 && c->alg.n <= 63 ? 2 : 1) << ") bch_nms_rc(const bchlib::NmsArgs a) {\n"
     << "  extern __shared__ __align__(16) unsigned char smem[];\n  bchlib::rc_persistent<" << msg
     << ">(a, reinterpret_cast<uint32_t *>(smem));\n}\n";
+  return o.str();
+}
+
+// The source of the row-by-row backward kernel (rc_backward.cuh).
+static std::string jit_rcb_source(const bch_code *c) {
+  std::ostringstream o, tab;
+  std::string calls, bwd;
+  emit_rc_tables(tab, c, 32, &calls, &bwd);
+  o << "#define BCH_JIT_QFRAC 0\n#define RC_FB 32\n#define RC_PC 0\n#define RCB_WARPS " << kRcbWarps << "\n#define RCB_ACC "
+    << kRcbAcc << "\n";
+  emit_prologue(o, 0, false);
+  o << "}  // namespace bchlib\n" << tab.str() << kRcLayoutText << "\n" << kRcDeviceText << "\n" << kRcBackwardText
+    << "\nnamespace bchlib {\n" << bwd << "}  // namespace bchlib\n"
+    << "extern \"C\" __global__ void __launch_bounds__(" << 32 * kRcbWarps
+    << ", 1) bch_bwd_rc(const bchlib::BwdArgs a) {\n"
+    << "  extern __shared__ __align__(16) float bwd_smem[];\n  bchlib::rcb_persistent(a, bwd_smem);\n}\n";
   return o.str();
 }
 
@@ -988,6 +1016,26 @@ cudaKernel_t jit_rc_kernel(const bch_code *c, int msg, int qfrac, int FB, int P,
   return k;
 }
 
+// The row-by-row backward kernel of code c; nullptr with *err when it does not compile.
+cudaKernel_t jit_rcb_kernel(const bch_code *c, std::string *err) {
+  {
+    std::lock_guard<std::mutex> lk(c->jit_mu);
+    for (const auto &m : c->jit_memo)
+      if (m.key == "rcb") {
+        if (!m.kernel) *err = m.err;
+        return static_cast<cudaKernel_t>(m.kernel);
+      }
+  }
+  std::string why;
+  cudaKernel_t k = compile_source(jit_rcb_source(c), "bch_bwd_rc", &why);
+  {
+    std::lock_guard<std::mutex> lk(c->jit_mu);
+    c->jit_memo.push_back({"rcb", static_cast<void *>(k), why});
+  }
+  if (!k) *err = why;
+  return k;
+}
+
 cudaKernel_t jit_serve_kernel(const bch_code *const *codes, int n_codes, std::string *err) {
   return compile_source(jit_serve_source(codes, n_codes), "bch_serve_jit", err);
 }
@@ -1005,6 +1053,14 @@ bool jit_compile_check(const bch_code *c, int msg, std::string *log) {
   for (int fb : {1, 32}) {  // the row/column kernels too
     std::string one;
     if (!compile_check_source(jit_rc_source(c, msg, 0, fb, 3), "bch_nms_rc", &one)) {
+      *log = one;
+      return false;
+    }
+    rc_log += one;
+  }
+  if (msg == 0) {  // and the backward kernel
+    std::string one;
+    if (!compile_check_source(jit_rcb_source(c), "bch_bwd_rc", &one)) {
       *log = one;
       return false;
     }

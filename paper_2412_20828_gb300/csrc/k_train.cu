@@ -192,6 +192,12 @@ __global__ void reduce_alpha_kernel(const float *partial, int nb, int I, float *
   }
 }
 
+cudaError_t launch_reduce_alpha(const float *partial, int nb, int I, float *grad_alpha, cudaStream_t st) {
+  note_launch();
+  reduce_alpha_kernel<<<I, 256, 0, st>>>(partial, nb, I, grad_alpha);
+  return cudaGetLastError();
+}
+
 template <int TPB, int WB>
 static cudaError_t launch_bwd_wb(const BwdArgs &a, int nb, size_t smem, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(nms_backward_kernel<TPB, WB>,
@@ -203,7 +209,7 @@ static cudaError_t launch_bwd_wb(const BwdArgs &a, int nb, size_t smem, cudaStre
 }
 
 size_t backward_workspace(int F, int I) {
-  const int nb = (F + 63) / 64;
+  const int nb = (F + 31) / 32;  // one partial per block: 32 frames (row by row) or 64
   return size_t(nb) * size_t(I) * sizeof(float);
 }
 
@@ -228,9 +234,7 @@ cudaError_t launch_backward(const BwdArgs &a0, float *grad_alpha, cudaStream_t s
   else
     e = cudaErrorNotSupported;
   if (e != cudaSuccess) return e;
-  note_launch();
-  reduce_alpha_kernel<<<a0.I, 256, 0, st>>>(a0.partial, nb, a0.I, grad_alpha);
-  return cudaGetLastError();
+  return launch_reduce_alpha(a0.partial, nb, a0.I, grad_alpha, st);
 }
 
 }  // namespace bchlib

@@ -58,4 +58,13 @@ inline RcLayout rc_layout(int n, int P, int R, int FB, int rs_words, int kw, int
   return L;
 }
 
+// Words of the backward kernel (rc_backward.cuh) with n_acc sums.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int rcb_words(int n, int P, int R, int w4, int warps, int n_acc) {
+  return ((3 * n * 33 + 3) & ~3) + 2 * n * 32 + R * 96 + n_acc * n * 32 + 32 + warps + 32 + P * 32 +
+         R * w4 * 2;
+}
+
 }  // namespace bchlib

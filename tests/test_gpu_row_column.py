@@ -2,7 +2,9 @@
 kernel: the same additions in the same order, so every output is bit-identical -- hard
 decisions, iterations, flags and the final LLRs -- for each message format, at batch sizes
 around the blocks' edges, for any number of copies, and on frames with ties, zeros, tiny
-and huge values, infinities and NaN.  (The other decode tests hold both to the oracle.)"""
+and huge values, infinities and NaN.  (The other decode tests hold both to the oracle.)
+The row-by-row backward kernel against the precompiled one: the same terms in another
+order, on the same kinds of frames."""
 import numpy as np
 import pytest
 
@@ -73,3 +75,37 @@ def test_checkpoints_bit_identical(nk, monkeypatch):
         B.nms_forward_train(code, B.params(iters, 0.7), to_dev(llr), autos_dev(autos), ck)
         got.append(ck)
     assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
+
+
+@pytest.mark.parametrize("nk", [(15, 7), (63, 45), (127, 64), (127, 99)])
+@pytest.mark.parametrize("F,P,iters,pad", [(1, 3, 4, 0), (33, 3, 6, 1), (500, 3, 12, 1), (65, 9, 3, 0)])
+def test_backward_against_precompiled(nk, F, P, iters, pad, monkeypatch):
+    """Both kernels add the same FP32 terms; each iteration's gradient is a chain of at most
+    (row weight + copies x column degree) additions, so their results differ by at most
+    iterations x that x 2^-24 of the gradient's norm (dL/dalpha: the oracle tests' 2e-3)."""
+    import torch
+    n, k = nk
+    code, ld = B.Code(n, k), n + pad
+    H = code.dense()
+    llr = _llr(n, k, F, ld, 800 + F)
+    autos = autos_dev(B.draw_automorphisms_host(n, P, 33, 0, F))
+    p = B.params(iters, 0.7, n_autos=P)
+    ck = torch.zeros((iters + 1, F, ld), device="cuda")
+    B.nms_forward_train(code, p, to_dev(llr), autos, ck)
+    go = torch.from_numpy(np.random.default_rng(F).standard_normal((F, ld)).astype(np.float32)).cuda()
+    got = []
+    for mode in ("generic", "auto"):
+        monkeypatch.setenv("BCHDEC_NMS_KERNEL", mode)
+        gl, ga = torch.zeros((F, ld), device="cuda"), torch.zeros(iters, device="cuda")
+        B.nms_backward(code, p, autos, ck, go, gl, ga)
+        got.append((gl[:, :n].double(), ga.double()))
+    (g0, a0), (g1, a1) = got
+    fine = torch.isfinite(g0)
+    assert torch.equal(fine, torch.isfinite(g1))
+    chain = int(H.sum(1).max()) + P * int(H.sum(0).max())
+    assert (g0 - g1)[fine].norm() <= iters * chain * 2.0 ** -24 * g0[fine].norm()
+    usable = torch.isfinite(a0) & torch.isfinite(a1)
+    assert torch.equal(usable, torch.isfinite(a0))
+    # against the largest factor's gradient: the terms of opposite sign cancel in the others
+    if usable.any():  # a frame of infinities makes every factor's gradient NaN
+        assert ((a0 - a1)[usable].abs() <= 2e-3 * a0[usable].abs().max()).all()
