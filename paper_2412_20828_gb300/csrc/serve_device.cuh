@@ -163,7 +163,9 @@ __device__ __forceinline__ void serve_loop(const SrvArgs &a, unsigned char *smem
   int slot = -1, f = -1, t = 0;   // this lane's frame
   const float invP = 1.0f / float(a.P);
   for (;;) {
-    if (a.sh->stop) break;
+    // lane 0 reads the flag and the clock for the whole warp: lanes that decided for
+    // themselves could part, and the warp's shuffles need all of them
+    if (__shfl_sync(kFull, lane == 0 ? int(a.sh->stop) : 0, 0)) break;
     // ---- an idle warp binds to a code with published work
     if (!__any_sync(kFull, f >= 0)) {
       int pick = -1;
@@ -178,7 +180,7 @@ __device__ __forceinline__ void serve_loop(const SrvArgs &a, unsigned char *smem
       }
       pick = __shfl_sync(kFull, pick, 0);
       if (pick < 0) {
-        if (globaltimer() - idle_since > a.idle_ns) break;
+        if (__shfl_sync(kFull, int(globaltimer() - idle_since > a.idle_ns), 0)) break;
         __nanosleep(sleep_ns);
         sleep_ns = sleep_ns < 20000 ? sleep_ns * 2 : sleep_ns;
         continue;
@@ -666,7 +668,7 @@ template <class Sessions>
 __device__ __forceinline__ void serve_blocks(const SrvArgs &a, unsigned char *smem, const Sessions &sessions) {
   const int P = a.P;
   const SrvBlockLayout L = srv_block_layout(a.blk_max_rows, a.blk_flat_n, P, a.blk_R, 127);
-  volatile int *ctl = reinterpret_cast<volatile int *>(smem);  // [0] claiming, [1] pick, [2] stop
+  volatile int *ctl = reinterpret_cast<volatile int *>(smem);  // [0] claiming, [1] pick, [2] leave
   float *alpha_s = reinterpret_cast<float *>(smem + L.alpha);
   uint4 *rowmask = reinterpret_cast<uint4 *>(smem + L.rowmask);
   const int tid = int(threadIdx.x);
@@ -688,15 +690,16 @@ __device__ __forceinline__ void serve_blocks(const SrvArgs &a, unsigned char *sm
           }
         }
       }
+      // one thread's clock decides for the block: threads that each compared their own could
+      // part at the limit, and a session's named barrier counts all of them
       ctl[1] = pick;
-      ctl[2] = stop;
+      ctl[2] = stop || (pick < 0 && globaltimer() - idle_since > a.idle_ns);
       ctl[0] = 1;
     }
     __syncthreads();
-    const int pick = ctl[1], stop = ctl[2];
-    if (stop) break;
+    const int pick = ctl[1], leave = ctl[2];
+    if (leave) break;
     if (pick < 0) {
-      if (globaltimer() - idle_since > a.idle_ns) break;
       __nanosleep(sleep_ns);
       sleep_ns = sleep_ns < 20000 ? sleep_ns * 2 : sleep_ns;
       __syncthreads();

@@ -226,3 +226,24 @@ def test_cancel_queued_in_flight_and_completed_requests(setup):
         assert np.array_equal(B.unpack_bits(got[rids[1]][0], n)[ok], ref["final"][ok])
     finally:
         srv.close()
+
+
+def test_idle_exit_between_bursts(setup):
+    """Bursts that arrive around the kernel's idle limit: a block leaves as a whole or not at
+    all (one thread's clock decides), so every burst completes with the same results."""
+    import time
+    torch, codes, stds = setup
+    srv = B.Server(codes, stds, 12, 0.78, budget_bytes=1 << 28, idle_exit_us=40)
+    try:
+        reqs = [(i, frames(n, k, 3 + i, 3.0, 900 + i, ld=n + 1)[1]) for i, (n, k) in enumerate(CODES)]
+        first = None
+        for burst in range(400):
+            rids = [srv.submit(i, llr, 5, 100 * i) for i, llr in reqs]
+            got = _drain(srv, rids)
+            out = [x for rid in rids for x in got[rid]]
+            first = first or out
+            assert all(np.array_equal(a, b) for a, b in zip(first, out)), burst
+            time.sleep((burst % 20) * 5e-6)
+        assert srv.stats()["completed"] == 400 * len(reqs)
+    finally:
+        srv.close()
