@@ -214,6 +214,76 @@ __device__ __forceinline__ int8_t int8_store_quotient(float N, int k, int d) {
   return int8_t(int8_quotient_exact(N, k, d));
 }
 
+// ---------------------------------------------------------------- two smallest of W values
+__device__ __forceinline__ float mn2(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float mx2(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ float mn3(float a, float b, float c) {
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ int mn2(int a, int b) { return min(a, b); }
+__device__ __forceinline__ int mx2(int a, int b) { return max(a, b); }
+__device__ __forceinline__ int mn3(int a, int b, int c) { return __vimin3_s32(a, b, c); }
+
+__host__ __device__ constexpr int grid_side(int W) {  // smallest a with a a >= W
+  int a = 1;
+  while (a * a < W) a++;
+  return a;
+}
+
+// min1 and min2 (with multiplicity) of W >= 2 values, none of them NaN.  A running pair
+// costs 3 min/max per value.  From 8 values on they are laid out as a grid: the smallest
+// value sits in one line and one column of it, and the second smallest is in another line
+// or in another column, so min2 is the smaller of the second smallest line minimum and the
+// second smallest column minimum: about 2.5 two-input operations per value, in short chains
+// (min.f32 with three inputs issues as two operations on sm_103a: 835 M warp instructions
+// of the straight-line rows become 800 M, not 690 M).
+template <class T, int W>
+__device__ __forceinline__ void min12(const T (&x)[W], T &m1, T &m2) {
+  if constexpr (W < 8) {
+    m1 = mn2(x[0], x[1]);
+    m2 = mx2(x[0], x[1]);
+#pragma unroll
+    for (int i = 2; i + 1 < W; i += 2) {
+      const T lo = mn2(x[i], x[i + 1]), hi = mx2(x[i], x[i + 1]);
+      m2 = mn3(m2, mx2(m1, lo), hi);
+      m1 = mn2(m1, lo);
+    }
+    if constexpr (W % 2) {
+      m2 = mn2(m2, mx2(m1, x[W - 1]));
+      m1 = mn2(m1, x[W - 1]);
+    }
+  } else {
+    constexpr int B = grid_side(W), A = (W + B - 1) / B;  // A lines of B
+    T line[A], col[B];
+#pragma unroll
+    for (int g = 0; g < A; g++) {
+      T v = x[g * B];
+#pragma unroll
+      for (int k = 1; k < B && g * B + k < W; k += 2) {
+        if (k + 1 < B && g * B + k + 1 < W) v = mn3(v, x[g * B + k], x[g * B + k + 1 < W ? g * B + k + 1 : 0]);
+        else v = mn2(v, x[g * B + k]);
+      }
+      line[g] = v;
+    }
+#pragma unroll
+    for (int k = 0; k < B; k++) {
+      T v = x[k];
+#pragma unroll
+      for (int g = 1; g < A && g * B + k < W; g += 2) {
+        if (g + 1 < A && (g + 1) * B + k < W) v = mn3(v, x[g * B + k], x[(g + 1) * B + k < W ? (g + 1) * B + k : 0]);
+        else v = mn2(v, x[g * B + k]);
+      }
+      col[k] = v;
+    }
+    T l2, c1, c2;
+    min12<T, A>(line, m1, l2);
+    min12<T, B>(col, c1, c2);
+    m2 = mn2(l2, c2);
+  }
+}
+
 // Shared-memory carve-up common to the NMS kernels.
 struct GroupDesc {
   int w, rows, off, pad;

@@ -10,8 +10,8 @@
 // those sums to the gradient position by position.  A per-edge column pass (as the forward
 // has) would read 12 bytes for each of a row's ~23 edges, of which two matter.
 //
-// Bound: the ALU pipe.  Per edge: an address, 1.85 three-input minima, half a sign xor and two
-// equality tests on it (2.7 SM cycles per 32 lanes), beside two shared-memory reads and
+// Bound: the ALU pipe.  Per edge: an address, 2.5 minima, half a sign xor and two equality
+// tests on it (3 SM cycles per 32 lanes), beside two shared-memory reads and
 // three additions.  BCH(127,64), 65 536 frames x 12 iterations x P = 3: 4.14 ms, against 45.0 ms
 // of the one-thread-per-frame kernel (rows from shared-memory tables, 64 threads and 98 KB
 // per block); per group of 32 frames and iteration the rows take ~39 k cycles (4.4 per
@@ -105,7 +105,7 @@ __device__ __forceinline__ void rcb_rows(RcbPtr &c, int nr, int r0, int t0) {
       sg ^= __float_as_uint(v[e]);
       av[e] = fabsf(v[e]);
     }
-    rc_min12<float, W>(av, m1, m2);
+    min12<float, W>(av, m1, m2);
     // Sums without the row's sign, which all terms share.  The edges of the two minima are
     // counted up on the FMA pipe (the ALU pipe bounds this loop): e1 = the one edge at min1,
     // e2 = 256 + the edge at min2, 512 or more when several are.

@@ -61,71 +61,6 @@ __device__ __forceinline__ typename RcV<MSG>::T rc_ld(const unsigned char *p) {
   return *reinterpret_cast<const typename RcV<MSG>::T *>(p);
 }
 
-// ---------------------------------------------------------------- two smallest of W values
-__device__ __forceinline__ float rc_mn(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ float rc_mx(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ float rc_mn3(float a, float b, float c) { return bch_min3f(a, b, c); }
-__device__ __forceinline__ int rc_mn(int a, int b) { return min(a, b); }
-__device__ __forceinline__ int rc_mx(int a, int b) { return max(a, b); }
-__device__ __forceinline__ int rc_mn3(int a, int b, int c) { return __vimin3_s32(a, b, c); }
-
-__host__ __device__ constexpr int rc_side(int W) {  // smallest a with a a >= W
-  int a = 1;
-  while (a * a < W) a++;
-  return a;
-}
-
-// min1 and min2 (with multiplicity) of W >= 2 values, none of them NaN.  A running pair
-// costs 3 min/max per value.  From 8 values on they are laid out as a grid: the smallest
-// value sits in one line and one column of it, and the second smallest is in another line
-// or in another column, so min2 is the smaller of the second smallest line minimum and the
-// second smallest column minimum: with three-input minima 1.9 operations per value at
-// W = 16 and 1.7 at W = 44, in short chains.
-template <class T, int W>
-__device__ __forceinline__ void rc_min12(const T (&x)[W], T &m1, T &m2) {
-  if constexpr (W < 8) {
-    m1 = rc_mn(x[0], x[1]);
-    m2 = rc_mx(x[0], x[1]);
-#pragma unroll
-    for (int i = 2; i + 1 < W; i += 2) {
-      const T lo = rc_mn(x[i], x[i + 1]), hi = rc_mx(x[i], x[i + 1]);
-      m2 = rc_mn3(m2, rc_mx(m1, lo), hi);
-      m1 = rc_mn(m1, lo);
-    }
-    if constexpr (W % 2) {
-      m2 = rc_mn(m2, rc_mx(m1, x[W - 1]));
-      m1 = rc_mn(m1, x[W - 1]);
-    }
-  } else {
-    constexpr int B = rc_side(W), A = (W + B - 1) / B;  // A lines of B
-    T line[A], col[B];
-#pragma unroll
-    for (int g = 0; g < A; g++) {
-      T v = x[g * B];
-#pragma unroll
-      for (int k = 1; k < B && g * B + k < W; k += 2) {
-        if (k + 1 < B && g * B + k + 1 < W) v = rc_mn3(v, x[g * B + k], x[g * B + k + 1 < W ? g * B + k + 1 : 0]);
-        else v = rc_mn(v, x[g * B + k]);
-      }
-      line[g] = v;
-    }
-#pragma unroll
-    for (int k = 0; k < B; k++) {
-      T v = x[k];
-#pragma unroll
-      for (int g = 1; g < A && g * B + k < W; g += 2) {
-        if (g + 1 < A && (g + 1) * B + k < W) v = rc_mn3(v, x[g * B + k], x[(g + 1) * B + k < W ? (g + 1) * B + k : 0]);
-        else v = rc_mn(v, x[g * B + k]);
-      }
-      col[k] = v;
-    }
-    T l2, c1, c2;
-    rc_min12<T, A>(line, m1, l2);
-    rc_min12<T, B>(col, c1, c2);
-    m2 = rc_mn(l2, c2);
-  }
-}
-
 // ---------------------------------------------------------------- rows
 // min1 / min2 of a row with infinities or NaN among its values, in the order of the
 // one-thread-per-frame kernels (fminf / fmaxf pass over a NaN, and a NaN edge lowers min2
@@ -242,7 +177,7 @@ __device__ __forceinline__ void rc_rows(const RcPtr &c, int nr, int r0, int t0) 
       for (int e = 0; e < W; e++) v[e] = rc_ld<MSG>(zr[e] + p * (kRcZP * 128));
 #pragma unroll
       for (int e = 0; e < W; e++) sg ^= rc_take(v[e]);
-      rc_min12<V, W>(v, m1, m2);
+      min12<V, W>(v, m1, m2);
       if constexpr (MSG == kFP32)
         if (c.slow) {
           const float2 o = rc_min12_ordered(c.z + p * (kRcZP * 128), W, [&](int e) {
@@ -333,10 +268,10 @@ __device__ __forceinline__ void rc_row_pass(const RcPtr &c) {
       V x0 = rc_ld<MSG>(z + (o.x & 0xffffu) * (RC_FB * 4)), x1 = rc_ld<MSG>(z + (o.x >> 16) * (RC_FB * 4));
       V x2 = rc_ld<MSG>(z + (o.y & 0xffffu) * (RC_FB * 4)), x3 = rc_ld<MSG>(z + (o.y >> 16) * (RC_FB * 4));
       sg ^= rc_take(x0) ^ rc_take(x1) ^ rc_take(x2) ^ rc_take(x3);
-      const V l0 = rc_mn(x0, x1), h0 = rc_mx(x0, x1), l1 = rc_mn(x2, x3), h1 = rc_mx(x2, x3);
-      const V lo = rc_mn(l0, l1), hi = rc_mn3(rc_mx(l0, l1), h0, h1);
-      m2 = rc_mn3(m2, rc_mx(m1, lo), hi);
-      m1 = rc_mn(m1, lo);
+      const V l0 = mn2(x0, x1), h0 = mx2(x0, x1), l1 = mn2(x2, x3), h1 = mx2(x2, x3);
+      const V lo = mn2(l0, l1), hi = mn3(mx2(l0, l1), h0, h1);
+      m2 = mn3(m2, mx2(m1, lo), hi);
+      m1 = mn2(m1, lo);
     }
     if constexpr (MSG == kFP32)
       if (c.slow) {
