@@ -53,7 +53,8 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
                           ("kAutosDeviceText", "autos_device.cuh"), ("kOsdDeviceText", "osd_device.cuh"),
                           ("kServeDeviceText", "serve_device.cuh"),
                           ("kRcLayoutText", "rc_layout.h"), ("kRcDeviceText", "rc_device.cuh"),
-                          ("kRcBackwardText", "rc_backward.cuh")):
+                          ("kRcBackwardText", "rc_backward.cuh"),
+                          ("kRcPlainText", "rc_plain.cuh")):
             with open(os.path.join(CSRC, name)) as g:
                 text = g.read()
             assert ")__BCHTEXT__" not in text

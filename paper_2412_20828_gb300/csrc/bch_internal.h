@@ -76,7 +76,7 @@ int gf2_rank(std::vector<Row> rows, int n);
 // Row/column kernels (rc_device.cuh): the lengths of the code's index tables.
 constexpr int kRcConstBytes = 60000;  // constant-memory tables of the 32-slot kernel
 struct RcTables {
-  int const_bytes = 0, rows16 = 0, cols16 = 0, kw = 0, w4 = 0;
+  int const_bytes = 0, rows16 = 0, cols16 = 0, kw = 0, w4 = 0, plain_cols = 0;
 };
 constexpr int kRcbWarps = 16, kRcbAcc = 4;  // backward kernel (rc_backward.cuh)
 int rc_threads(int slots, int tasks);

@@ -21,6 +21,7 @@ namespace bchlib {
 cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac = 0);
 cudaKernel_t jit_rc_kernel(const bch_code *c, int msg, int qfrac, int FB, int P, std::string *err);
 cudaKernel_t jit_rcb_kernel(const bch_code *c, std::string *err);
+cudaKernel_t jit_rcp_kernel(const bch_code *c, int FB, std::string *err);
 bool jit_compile_check(const bch_code *c, int msg, std::string *log);
 bool jit_serve_compile_check(const bch_code *const *codes, int n_codes, std::string *log);
 int jit_block_size(int n);
@@ -574,6 +575,7 @@ bch_status bch_nms_jit_check(int n, int k, int m_rows, uint64_t seed, const bch_
   bch_code c;
   bch_status s = build_host(n, k, BCH_PCM_OPTIMIZED, m_rows, seed, opts, &c);
   if (s != BCH_OK) return s;
+  c.rc = rc_tables(&c);
   std::string text;
   const bool ok = jit_compile_check(&c, msg, &text);
   std::snprintf(log, capacity, "%s", text.c_str());
@@ -760,9 +762,62 @@ static cudaError_t launch_rc(cudaKernel_t k, int FB, const bch_code *code, const
   return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
 }
 
+// ---- plain decoder (rc_plain.cuh)
+static size_t rcp_smem_bytes(const bch_code *code, int FB) {
+  const int R = int(code->rows.size());
+  return size_t(rcp_layout(code->alg.n, R, code->rc.w4, FB, code->rc.kw, 4 * code->rc.w4 * R, code->rc.plain_cols)
+                    .words) * 4;
+}
+
+// Frame slots per block (1, 16 or 32) of the plain decoder's kernel, or 0 for the precompiled
+// one.  BCHDEC_JIT_RC=0|1|16|32 overrides.  us for 8 iterations at 3 dB on the standard matrix,
+// precompiled / 1 / 16 / 32 slots: BCH(63,36) 500 frames 369 / 21 / 29 / 37, 2400 frames 372 /
+// 42 / 29 / 37, 10 000 frames 373 / 116 / 90 / 66, 200 000 frames 3173 / 1911 / 1320 / 952;
+// BCH(127,64) (32 frames' messages exceed shared memory) 1200 frames 1569 / 58 / 86, 2400
+// frames 1587 / 117 / 86, 50 000 frames 9392 / 1761 / 1738; BCH(127,99) 50 000 frames 4446 / 2158 /
+// 1030 / 776.
+static int rcp_slots(const bch_code *code, const NmsArgs &a, int sms) {
+  // a matrix too large for the precompiled kernel's state stays refused (by its launch)
+  if (nms_table_bytes_host(code->dc) + size_t(3 * code->alg.n + 5 * code->dc.rows) * 4 * 64 > 227 * 1024) return 0;
+  auto fits = [&](int FB) {
+    return rcp_smem_bytes(code, FB) <= 227 * 1024 && code->rows.size() * 4 * size_t(code->rc.w4) < 65535;
+  };
+  if (const char *v = std::getenv("BCHDEC_JIT_RC")) {
+    const int fb = std::atoi(v);
+    return (fb == 1 || fb == 16 || fb == 32) && fits(fb) ? fb : 0;
+  }
+  if (a.F <= sms * 8 && fits(1)) return 1;
+  if (a.F <= sms * 16 && fits(16)) return 16;
+  return fits(32) ? 32 : fits(16) ? 16 : fits(1) ? 1 : 0;
+}
+
+static cudaError_t launch_rcp(cudaKernel_t k, int FB, const bch_code *code, const NmsArgs &a, cudaStream_t st) {
+  const void *fn = reinterpret_cast<const void *>(k);
+  const size_t smem = rcp_smem_bytes(code, FB);
+  const int tpb = rc_threads(FB == 1 ? 1 : 32, std::max(code->alg.n, int(code->rows.size())));
+  int sms = 0, per_sm = 0;
+  cudaError_t e = launch_geometry(fn, tpb, smem, &sms, &per_sm);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const long long need = (a.F + FB - 1) / FB, blocks = std::min<long long>(need, (long long)sms * per_sm);
+  void *args[] = {const_cast<NmsArgs *>(&a)};
+  note_launch();
+  return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
+}
+
 static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaStream_t st,
                                    std::string *why) {
   const int mode = kernel_mode();
+  if (a.P == 0 && mode != 1) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int fb = rcp_slots(code, a, sms);
+    std::string err;
+    if (fb)
+      if (cudaKernel_t k = jit_rcp_kernel(code, fb, &err)) return launch_rcp(k, fb, code, a, st);
+  }
   if (a.P > 0 && mode != 1) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);

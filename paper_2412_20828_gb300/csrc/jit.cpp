@@ -43,6 +43,7 @@ extern const char kServeDeviceText[];
 extern const char kRcLayoutText[];
 extern const char kRcDeviceText[];
 extern const char kRcBackwardText[];
+extern const char kRcPlainText[];
 
 namespace {
 
@@ -686,6 +687,7 @@ static RcTables emit_rc_tables(std::ostringstream &o, const bch_code *c, int FB,
   info.w4 = int(w4);
   info.rows16 = int(w4 * M * 4);
   info.cols16 = int(4 * size_t((n + 1) / 2) + d4 * n * 4);
+  info.plain_cols = info.cols16;  // the same degrees, message indices instead of row states
   std::ostringstream rows, cols, rcalls, ccalls, bcalls;
   size_t rt = 0, ct = 0;
   for (int i = 0; i < M;) {
@@ -793,6 +795,59 @@ static std::string jit_rcb_source(const bch_code *c) {
     << "extern \"C\" __global__ void __launch_bounds__(" << 32 * kRcbWarps
     << ", 1) bch_bwd_rc(const bchlib::BwdArgs a) {\n"
     << "  extern __shared__ __align__(16) float bwd_smem[];\n  bchlib::rcb_persistent(a, bwd_smem);\n}\n";
+  return o.str();
+}
+
+// The source of the plain decoder's kernel (rc_plain.cuh) with FB slots.  Rows in the order of
+// the precompiled kernel's groups (by weight, stable), which is the order of its additions.
+static std::string jit_rcp_source(const bch_code *c, int FB) {
+  const int n = c->alg.n, M = int(c->rows.size()), w4 = c->rc.w4, kw = c->rc.kw, K = int(c->alg.std_h.size());
+  std::vector<int> order(M), corder(n);
+  for (int i = 0; i < M; i++) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return c->rows[a].weight() < c->rows[b].weight(); });
+  std::vector<std::vector<int>> by_row(M), by_col(n);
+  for (int i = 0; i < M; i++)
+    for (int u = 0; u < n; u++)
+      if (c->rows[order[i]].get(u)) {
+        by_col[u].push_back(i * 4 * w4 + int(by_row[i].size()));
+        by_row[i].push_back(u);
+      }
+  size_t d4 = 0;
+  for (int u = 0; u < n; u++) {
+    corder[u] = u;
+    while (by_col[u].size() % 4) by_col[u].push_back(M * 4 * w4);
+    d4 = std::max(d4, by_col[u].size() / 4);
+  }
+  std::stable_sort(corder.begin(), corder.end(), [&](int a, int b) { return by_col[a].size() > by_col[b].size(); });
+  std::ostringstream o;
+  o << "#define BCH_JIT_QFRAC 0\n#define RC_FB " << FB << "\n#define RC_N " << n << "\n#define RC_R " << M
+    << "\n#define RC_KW " << kw << "\n#define RC_W4 " << w4 << "\n#define RCP_ROWS " << 4 * w4 * M << "\n#define RCP_COLS "
+    << c->rc.plain_cols << "\n";
+  emit_prologue(o, 0, false);
+  o << "}  // namespace bchlib\n__device__ const uint32_t rc_cmask[] = {";
+  for (int u = 0; u < n; u++)
+    for (int w = 0; w < kw; w++) {
+      uint32_t v = 0;
+      for (int r = 32 * w; r < std::min(K, 32 * w + 32); r++) v |= uint32_t(c->alg.std_h[r].get(u)) << (r - 32 * w);
+      o << v << "u,";
+    }
+  o << "};\n__device__ __align__(16) const unsigned short rcp_rows[] = {";
+  for (int q = 0; q < w4; q++)
+    for (int r = 0; r < M; r++)
+      for (size_t h = 4 * q; h < size_t(4 * q + 4); h++) o << (h < by_row[r].size() ? by_row[r][h] : n) << ",";
+  o << "};\n__device__ __align__(16) const unsigned short rcp_cols[] = {";
+  for (int i = 0; i < 2 * ((n + 1) / 2); i++)
+    o << (i < n ? corder[i] : 0) << "," << (i < n ? by_col[corder[i]].size() / 4 : 0) << ",";
+  for (size_t q = 0; q < d4; q++)
+    for (int i = 0; i < n; i++)
+      for (size_t h = 4 * q; h < 4 * q + 4; h++) {
+        const auto &v = by_col[corder[i]];
+        o << (h < v.size() ? v[h] : M * 4 * w4) << ",";
+      }
+  o << "};\n" << kRcLayoutText << "\n" << kRcPlainText << "\n"
+    << "extern \"C\" __global__ void __launch_bounds__(512, 1) bch_plain_rc(const bchlib::NmsArgs a) {\n"
+    << "  extern __shared__ __align__(16) unsigned char smem[];\n"
+    << "  bchlib::rcp_persistent(a, reinterpret_cast<uint32_t *>(smem));\n}\n";
   return o.str();
 }
 
@@ -1058,6 +1113,27 @@ cudaKernel_t jit_rcb_kernel(const bch_code *c, std::string *err) {
   return k;
 }
 
+// The plain decoder's kernel of code c with FB slots; nullptr with *err when it does not compile.
+cudaKernel_t jit_rcp_kernel(const bch_code *c, int FB, std::string *err) {
+  const std::string key = "rcp/" + std::to_string(FB);
+  {
+    std::lock_guard<std::mutex> lk(c->jit_mu);
+    for (const auto &m : c->jit_memo)
+      if (m.key == key) {
+        if (!m.kernel) *err = m.err;
+        return static_cast<cudaKernel_t>(m.kernel);
+      }
+  }
+  std::string why;
+  cudaKernel_t k = compile_source(jit_rcp_source(c, FB), "bch_plain_rc", &why);
+  {
+    std::lock_guard<std::mutex> lk(c->jit_mu);
+    c->jit_memo.push_back({key, static_cast<void *>(k), why});
+  }
+  if (!k) *err = why;
+  return k;
+}
+
 cudaKernel_t jit_serve_kernel(const bch_code *const *codes, int n_codes, std::string *err) {
   return compile_source(jit_serve_source(codes, n_codes), "bch_serve_jit", err);
 }
@@ -1080,8 +1156,13 @@ bool jit_compile_check(const bch_code *c, int msg, std::string *log) {
     }
     rc_log += one;
   }
-  if (msg == 0) {  // and the backward kernel
+  if (msg == 0) {  // and the plain and backward kernels
     std::string one;
+    if (!compile_check_source(jit_rcp_source(c, 32), "bch_plain_rc", &one)) {
+      *log = one;
+      return false;
+    }
+    rc_log += one;
     if (!compile_check_source(jit_rcb_source(c), "bch_bwd_rc", &one)) {
       *log = one;
       return false;

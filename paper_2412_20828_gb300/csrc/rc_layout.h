@@ -58,6 +58,41 @@ inline RcLayout rc_layout(int n, int P, int R, int FB, int rs_words, int kw, int
   return L;
 }
 
+// The plain decoder's kernel (rc_plain.cuh): channel values and totals (with a padded edge's
+// value), messages (with a neutral one), the tables.
+struct RcpLayout {
+  int ch, x, msg, synd, f, alpha, cmask, rows, cols, words;
+};
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline RcpLayout rcp_layout(int n, int R, int w4, int FB, int kw, int tab_rows, int tab_cols) {
+  RcpLayout L;
+  int o = 0;
+  L.ch = o;
+  o += n * (FB == 32 ? 33 : FB);
+  L.x = o;
+  o += (n + 1) * FB;
+  L.msg = o;
+  o += (R * 4 * w4 + 1) * FB;
+  L.synd = o;
+  o += kw * FB;
+  L.f = o;
+  o += FB;
+  L.alpha = o;
+  o += 32;
+  L.cmask = o;
+  o += kw * n;
+  o = (o + 1) & ~1;
+  L.rows = o;
+  o += (tab_rows + 1) / 2;
+  o = (o + 1) & ~1;
+  L.cols = o;
+  o += (tab_cols + 1) / 2;
+  L.words = o;
+  return L;
+}
+
 // Words of the backward kernel (rc_backward.cuh) with n_acc sums.
 #ifdef __CUDACC__
 __host__ __device__

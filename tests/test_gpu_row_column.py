@@ -3,6 +3,7 @@ kernel: the same additions in the same order, so every output is bit-identical -
 decisions, iterations, flags and the final LLRs -- for each message format, at batch sizes
 around the blocks' edges, for any number of copies, and on frames with ties, zeros, tiny
 and huge values, infinities and NaN.  (The other decode tests hold both to the oracle.)
+The plain decoder's kernel against the precompiled one likewise.
 The row-by-row backward kernel against the precompiled one: the same terms in another
 order, on the same kinds of frames."""
 import numpy as np
@@ -59,6 +60,26 @@ def test_bit_identical_to_one_thread_per_frame(nk, kw, monkeypatch):
             got = _decode(monkeypatch, rc, code, llr, autos, iters, kk)
             for name, x, y in zip(("hard", "iters", "flags", "llr"), ref, got):
                 assert np.array_equal(x, y), (name, F, P, iters, rc)
+
+
+@pytest.mark.parametrize("nk", [(15, 7), (63, 36), (127, 64), (127, 99)])
+def test_plain_bit_identical_to_precompiled(nk, monkeypatch):
+    import torch
+    n, k = nk
+    code = B.Code(n, k, kind=B.PCM_STANDARD)
+    for F, iters, stop, ld in ((1, 8, True, n), (33, 8, True, n + 1), (700, 10, False, n + 1), (9000, 8, True, n)):
+        llr, got = to_dev(_llr(n, k, F, ld, 700 + F)), []
+        for rc in ("generic", "1", "16", "32"):
+            monkeypatch.setenv("BCHDEC_NMS_KERNEL", "generic" if rc == "generic" else "auto")
+            monkeypatch.setenv("BCHDEC_JIT_RC", rc)
+            out = [torch.full((F, (n + 63) // 64), -1, dtype=torch.int64, device="cuda"),
+                   torch.zeros(F, dtype=torch.uint8, device="cuda"),
+                   torch.full((F,), 9, dtype=torch.uint8, device="cuda"), torch.zeros((F, ld), device="cuda")]
+            B.nms_decode(code, B.params(iters, 0.78, n_autos=0, early_stop=stop), llr, None, *out)
+            got.append([o.cpu().numpy().view(np.uint8) for o in out])
+        for rc in (1, 2, 3):
+            for name, x, y in zip(("hard", "iters", "flags", "llr"), got[0], got[rc]):
+                assert np.array_equal(x, y), (name, F, rc)
 
 
 @pytest.mark.parametrize("nk", [(63, 45), (127, 64)])
