@@ -56,8 +56,10 @@ unsigned *check_word();
 cudaError_t launch_geometry(const void *fn, int tpb, size_t smem, int *sms, int *per_sm);
 cudaError_t launch_nms(const NmsArgs &a, cudaStream_t st);
 cudaError_t launch_osd(const OsdArgs &a, cudaStream_t st);
+// With few frames (compact_clears_queue) one launch, which also clears *queue (nullable).
+bool compact_clears_queue(int F);
 cudaError_t launch_compact(const uint8_t *flags, int F, uint32_t *counts, uint32_t *list,
-                           uint32_t *count, cudaStream_t st);
+                           uint32_t *count, unsigned *queue, cudaStream_t st);
 cudaError_t launch_draw_autos(int n, int ord, int P, uint64_t seed, uint64_t frame0, int F,
                               uint16_t *out, cudaStream_t st);
 cudaError_t launch_gen_frames(const GenArgs &a, cudaStream_t st);

@@ -707,6 +707,12 @@ static cudaError_t launch_jit(cudaKernel_t k, const bch_code *code, const NmsArg
   return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
 }
 
+// Zeroes the workspace's queue counters (the min-sum kernel's frame queue, the OSD's).
+static cudaError_t clear_queue(const NmsArgs &a, cudaStream_t st, bool *cleared) {
+  *cleared = true;
+  return cudaMemsetAsync(a.queue, 0, 16, st);
+}
+
 // ---- row/column kernels (rc_device.cuh)
 static size_t rc_smem_bytes(const bch_code *code, const NmsArgs &a, int FB) {
   return size_t(rc_layout(code->alg.n, a.P, int(code->rows.size()), FB, a.msg == BCH_MSG_INT8 ? 3 : 2,
@@ -748,7 +754,8 @@ static int rc_slots(const bch_code *code, const NmsArgs &a, int sms) {
   return !cached || a.F <= sms * many ? 32 : 0;
 }
 
-static cudaError_t launch_rc(cudaKernel_t k, int FB, const bch_code *code, const NmsArgs &a, cudaStream_t st) {
+static cudaError_t launch_rc(cudaKernel_t k, int FB, const bch_code *code, const NmsArgs &a, cudaStream_t st,
+                             bool *cleared) {
   const void *fn = reinterpret_cast<const void *>(k);
   const size_t smem = rc_smem_bytes(code, a, FB);
   const int tpb = rc_threads(FB, a.P * std::max(code->alg.n, int(code->rows.size())));
@@ -757,6 +764,10 @@ static cudaError_t launch_rc(cudaKernel_t k, int FB, const bch_code *code, const
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long need = (a.F + FB - 1) / FB, blocks = std::min<long long>(need, (long long)sms * per_sm);
+  if (blocks < need) {  // the blocks' first frames are fixed; only later ones come from the queue
+    e = clear_queue(a, st, cleared);
+    if (e != cudaSuccess) return e;
+  }
   void *args[] = {const_cast<NmsArgs *>(&a)};
   note_launch();
   return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
@@ -791,7 +802,8 @@ static int rcp_slots(const bch_code *code, const NmsArgs &a, int sms) {
   return fits(32) ? 32 : fits(16) ? 16 : fits(1) ? 1 : 0;
 }
 
-static cudaError_t launch_rcp(cudaKernel_t k, int FB, const bch_code *code, const NmsArgs &a, cudaStream_t st) {
+static cudaError_t launch_rcp(cudaKernel_t k, int FB, const bch_code *code, const NmsArgs &a, cudaStream_t st,
+                              bool *cleared) {
   const void *fn = reinterpret_cast<const void *>(k);
   const size_t smem = rcp_smem_bytes(code, FB);
   const int tpb = rc_threads(FB == 1 ? 1 : 32, std::max(code->alg.n, int(code->rows.size())));
@@ -800,13 +812,18 @@ static cudaError_t launch_rcp(cudaKernel_t k, int FB, const bch_code *code, cons
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long need = (a.F + FB - 1) / FB, blocks = std::min<long long>(need, (long long)sms * per_sm);
+  if (blocks < need) {  // the blocks' first frames are fixed; only later ones come from the queue
+    e = clear_queue(a, st, cleared);
+    if (e != cudaSuccess) return e;
+  }
   void *args[] = {const_cast<NmsArgs *>(&a)};
   note_launch();
   return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
 }
 
+// Launches the min-sum kernel for this call; *cleared: whether the queue counters were zeroed.
 static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaStream_t st,
-                                   std::string *why) {
+                                   std::string *why, bool *cleared) {
   const int mode = kernel_mode();
   if (a.P == 0 && mode != 1) {
     int dev = 0, sms = 0;
@@ -816,7 +833,7 @@ static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaS
     const int fb = rcp_slots(code, a, sms);
     std::string err;
     if (fb)
-      if (cudaKernel_t k = jit_rcp_kernel(code, fb, &err)) return launch_rcp(k, fb, code, a, st);
+      if (cudaKernel_t k = jit_rcp_kernel(code, fb, &err)) return launch_rcp(k, fb, code, a, st, cleared);
   }
   if (a.P > 0 && mode != 1) {
     int dev = 0, sms = 0;
@@ -826,8 +843,10 @@ static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaS
     const int fb = rc_slots(code, a, sms);
     std::string err;
     if (fb)
-      if (cudaKernel_t k = jit_rc_kernel(code, a.msg, a.qfrac, fb, a.P, &err)) return launch_rc(k, fb, code, a, st);
+      if (cudaKernel_t k = jit_rc_kernel(code, a.msg, a.qfrac, fb, a.P, &err)) return launch_rc(k, fb, code, a, st, cleared);
   }
+  const cudaError_t ec = clear_queue(a, st, cleared);
+  if (ec != cudaSuccess) return ec;
   // auto and jit: the specialised kernel (for n = 127 it spills but still runs 1.8x
   // faster than the precompiled one; its first compile takes tens of seconds and is
   // cached on disk); auto falls back to the precompiled kernel if it does not compile
@@ -871,7 +890,7 @@ static cudaError_t launch_backward_code(const bch_code *code, const BwdArgs &a, 
 static bch_status run_nms(const bch_code *code, const bch_nms_params *params, const float *llr, int ld,
                           int n_frames, const uint16_t *autos, uint64_t *hard, uint8_t *iters,
                           uint8_t *flags, float *llr_out, float *ckpt, void *workspace,
-                          cudaStream_t st) {
+                          cudaStream_t st, bool *queue_cleared = nullptr) {
   bch_status s = check_params(code, params);
   if (s != BCH_OK) return s;
   s = check_frames(code, llr, ld, n_frames);
@@ -883,11 +902,12 @@ static bch_status run_nms(const bch_code *code, const bch_nms_params *params, co
   const WsLayout L = ws_layout(n_frames, params->iters);
   unsigned char *ws = static_cast<unsigned char *>(workspace);
   unsigned *queue = reinterpret_cast<unsigned *>(ws + L.queues);
-  BCH_CUDA(cudaMemsetAsync(queue, 0, 16, st), "clear queue");
   NmsArgs a = make_nms_args(code, params, llr, ld, n_frames, autos, hard, iters, flags, llr_out, queue);
   a.ckpt = ckpt;
   std::string why;
-  cudaError_t e = launch_nms_code(code, a, st, &why);
+  bool cleared = false;
+  cudaError_t e = launch_nms_code(code, a, st, &why, &cleared);
+  if (queue_cleared) *queue_cleared = cleared;
   if (e != cudaSuccess) return fail(BCH_ECUDA, std::string("nms kernel: ") + cudaGetErrorString(e) + " " + why);
   return BCH_OK;
 }
@@ -952,16 +972,18 @@ bch_status bch_hybrid_decode(const bch_code *code, const bch_code *std_code, con
   if (s != BCH_OK) return s;
   if (params->osd_input == 1 && !llr_out)
     return fail(BCH_EINVAL, "osd_input = 1 needs llr_out (the NMS output the OSD reads)");
+  bool cleared = false;
   s = run_nms(code, params, llr, ld, n_frames, autos, hard, iters, flags, llr_out, nullptr,
-                         workspace, st);
+                         workspace, st, &cleared);
   if (s != BCH_OK || n_frames == 0) return s;
   const WsLayout L = ws_layout(n_frames, params->iters);
   unsigned char *ws = static_cast<unsigned char *>(workspace);
   uint32_t *list = failed_list ? failed_list : reinterpret_cast<uint32_t *>(ws + L.list);
   uint32_t *count = failed_count ? failed_count : reinterpret_cast<uint32_t *>(ws + L.count);
-  BCH_CUDA(launch_compact(flags, n_frames, reinterpret_cast<uint32_t *>(ws + L.counts), list, count, st),
-           "compaction");
   unsigned *queue = reinterpret_cast<unsigned *>(ws + L.queues);
+  if (!cleared && !compact_clears_queue(n_frames)) BCH_CUDA(cudaMemsetAsync(queue, 0, 16, st), "clear queue");
+  BCH_CUDA(launch_compact(flags, n_frames, reinterpret_cast<uint32_t *>(ws + L.counts), list, count, queue + 1, st),
+           "compaction");
   if (params->osd_input == 1)  // the failed frames' final y, scaled per frame in the OSD
     return run_osd(std_code, params->osd_order, llr_out, ld, list, count, n_frames, hard, flags, queue + 1,
                    st, 1);
@@ -976,7 +998,7 @@ bch_status bch_compact_failed(const uint8_t *flags, int n_frames, uint32_t *list
   const WsLayout L = ws_layout(n_frames, 1);
   BCH_CUDA(launch_compact(flags, n_frames,
                           reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(workspace) + L.counts),
-                          list, count, static_cast<cudaStream_t>(stream)),
+                          list, count, nullptr, static_cast<cudaStream_t>(stream)),
            "compaction");
   return BCH_OK;
 }

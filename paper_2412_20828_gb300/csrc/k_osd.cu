@@ -101,9 +101,61 @@ __global__ void __launch_bounds__(kCompactBlock)
   }
 }
 
+// Compaction of up to kCompactSmall frames by one block, in one launch: every thread holds
+// its flags in registers.  It also clears *queue (the OSD's), which spares a small call the
+// memset.  Two launches and a memset took 9 us of a 32 us call of 7 frames.
+constexpr int kCompactSmall = 8 * kCompactBlock;
+
+__global__ void __launch_bounds__(kCompactBlock)
+    compact_small_kernel(const uint8_t *flags, int F, uint32_t *list, uint32_t *count, unsigned *queue) {
+  constexpr int kPer = kCompactSmall / kCompactBlock;
+  __shared__ uint32_t warp_cnt[kPer][kCompactBlock / 32];
+  __shared__ uint32_t total;
+  const int tid = int(threadIdx.x), warp = tid >> 5, lane = tid & 31;
+  unsigned b[kPer];
+#pragma unroll
+  for (int c = 0; c < kPer; c++) {
+    const int f = c * kCompactBlock + tid;
+    b[c] = __ballot_sync(kFull, f < F && !(flags[f] & BCH_FLAG_CONVERGED));
+    if (lane == 0) warp_cnt[c][warp] = __popc(b[c]);
+  }
+  __syncthreads();
+  if (warp == 0) {  // exclusive sums over (chunk, warp) in frame order
+    uint32_t base = 0;
+#pragma unroll
+    for (int c = 0; c < kPer; c++) {
+      const uint32_t v = warp_cnt[c][lane];
+      uint32_t inc = v;
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t u = __shfl_up_sync(kFull, inc, off);
+        if (lane >= off) inc += u;
+      }
+      warp_cnt[c][lane] = base + inc - v;
+      base += __shfl_sync(kFull, inc, 31);
+    }
+    if (lane == 0) total = base;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < kPer; c++)
+    if ((b[c] >> lane) & 1u)
+      list[warp_cnt[c][warp] + __popc(b[c] & ((1u << lane) - 1u))] = uint32_t(c * kCompactBlock + tid);
+  if (tid == 0) {
+    *count = total;
+    if (queue) *queue = 0u;
+  }
+}
+
+bool compact_clears_queue(int F) { return F > 0 && F <= kCompactSmall; }
+
 cudaError_t launch_compact(const uint8_t *flags, int F, uint32_t *counts, uint32_t *list,
-                           uint32_t *count, cudaStream_t st) {
+                           uint32_t *count, unsigned *queue, cudaStream_t st) {
   if (F <= 0) return cudaMemsetAsync(count, 0, sizeof(uint32_t), st);
+  if (compact_clears_queue(F)) {
+    note_launch();
+    compact_small_kernel<<<1, kCompactBlock, 0, st>>>(flags, F, list, count, queue);
+    return cudaGetLastError();
+  }
   const int nb = (F + kCompactBlock - 1) / kCompactBlock;
   note_launch();
   count_failed_kernel<<<nb, kCompactBlock, 0, st>>>(flags, F, counts);

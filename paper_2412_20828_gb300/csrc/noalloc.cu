@@ -142,7 +142,7 @@ extern "C" bch_status bch_hybrid_decode_noalloc(const bch_code *code, const bch_
   uint32_t *counts = reinterpret_cast<uint32_t *>(ws + kCountsOff);
   uint32_t *list = reinterpret_cast<uint32_t *>(ws + kListOff);
   uint32_t *count = reinterpret_cast<uint32_t *>(ws + kCountOff);
-  e = launch_compact(flags, n_frames, counts, list, count, st);
+  e = launch_compact(flags, n_frames, counts, list, count, nullptr, st);
   if (e != cudaSuccess) return fail(BCH_ECUDA, std::string("compaction: ") + cudaGetErrorString(e));
 
   const int n = std_code->alg.n, M = n - std_code->alg.k;
