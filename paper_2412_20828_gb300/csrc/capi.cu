@@ -18,7 +18,8 @@
 using namespace bchlib;
 
 namespace bchlib {
-cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac = 0);
+cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac = 0, bool may_defer = true);
+bool jit_defers(int n, int msg);
 cudaKernel_t jit_rc_kernel(const bch_code *c, int msg, int qfrac, int FB, int P, std::string *err);
 cudaKernel_t jit_rcb_kernel(const bch_code *c, std::string *err);
 cudaKernel_t jit_rcp_kernel(const bch_code *c, int FB, std::string *err);
@@ -764,7 +765,7 @@ static cudaError_t launch_rc(cudaKernel_t k, int FB, const bch_code *code, const
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long need = (a.F + FB - 1) / FB, blocks = std::min<long long>(need, (long long)sms * per_sm);
-  if (blocks < need) {  // the blocks' first frames are fixed; only later ones come from the queue
+  if (blocks < need && !a.list) {  // the blocks' first frames are fixed; only later ones come from the queue
     e = clear_queue(a, st, cleared);
     if (e != cudaSuccess) return e;
   }
@@ -852,8 +853,20 @@ static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaS
   // cached on disk); auto falls back to the precompiled kernel if it does not compile
   if (a.P > 0 && mode != 1) {
     std::string err;
-    cudaKernel_t k = jit_kernel(code, a.msg, &err, a.qfrac);
-    if (k) return launch_jit(k, code, a, st);
+    // the FP32 kernel of n <= 63 leaves frames with an infinity or NaN to the row/column
+    // kernel, launched over its list (empty in all but odd calls: 2 us)
+    cudaKernel_t rk = nullptr;
+    if (jit_defers(code->alg.n, a.msg) && rc_fits(code, a, 1)) rk = jit_rc_kernel(code, a.msg, a.qfrac, 1, a.P, &err);
+    cudaKernel_t k = jit_kernel(code, a.msg, &err, a.qfrac, rk != nullptr);
+    if (k) {
+      cudaError_t e = launch_jit(k, code, a, st);
+      if (e != cudaSuccess || !rk) return e;
+      NmsArgs d = a;
+      d.list = a.defer;
+      d.list_count = a.defer_count;
+      d.queue = a.queue + 3;
+      return launch_rc(rk, 1, code, d, st, cleared);
+    }
     if (why) *why = err;
     if (mode == 2) return cudaErrorNotSupported;
   }
@@ -904,6 +917,10 @@ static bch_status run_nms(const bch_code *code, const bch_nms_params *params, co
   unsigned *queue = reinterpret_cast<unsigned *>(ws + L.queues);
   NmsArgs a = make_nms_args(code, params, llr, ld, n_frames, autos, hard, iters, flags, llr_out, queue);
   a.ckpt = ckpt;
+  // queue words: [0] frame queue, [1] the OSD's, [2] deferred frames, [3] their queue; the list
+  // shares the failed frames' space, which the compaction fills later
+  a.defer = reinterpret_cast<uint32_t *>(ws + L.list);
+  a.defer_count = queue + 2;
   std::string why;
   bool cleared = false;
   cudaError_t e = launch_nms_code(code, a, st, &why, &cleared);

@@ -330,15 +330,20 @@ static void emit_chain_loop(std::ostringstream &o, int n, const std::string &stm
 // us for 10^6 frames, Eb/N0 U[1, 6) dB, 0 / 1 / 2: FP16 BCH(63,36) 5863 / 5410 / 5541, (63,45)
 // 2568 / 2428 / 2420; INT8 (63,36) 5914 / 5527 / 5257, (63,45) 2942 / 2859 / 2747; with 8 fractional
 // bits 6049 / 5779 / 5654 and 2991 / 2859 / 2879.  BCHDEC_JIT_GRID=0 restores the edge order.
-// FP32 rows keep the edge order: a NaN among their values is passed over by position.
-static int jit_grid(int msg, int n) {
+// FP32 (0 / 1 / 2): (63,36) 3353 / 3119 / 3239, (63,45) 1837 / 1752 / 1746; a NaN is passed over by
+// its position in the edge order, so the batch kernel then defers frames with one (defer;
+// the serving kernels, which cannot, keep the edge order).
+static int jit_grid(int msg, int n, bool defer) {
   if (n > 63 || !jit_incr() || env_int("BCHDEC_JIT_GRID", 0, 1, 1) == 0) return 0;
-  return msg == 1 ? 1 : msg == 2 ? 2 : 0;
+  return msg == 1 ? 1 : msg == 2 ? 2 : defer ? 1 : 0;
 }
+// Whether the batch kernel of format msg defers frames (see jit_grid).
+bool jit_defers(int n, int msg) { return msg == 0 && jit_grid(0, n, true) != 0; }
 
-static void emit_copy_body(std::ostringstream &o, const bch_code *c, int msg, int stride, bool scratch) {
+static void emit_copy_body(std::ostringstream &o, const bch_code *c, int msg, int stride, bool scratch,
+                           bool defer = false) {
   const int n = c->alg.n, m = c->alg.m;
-  const int nw = (n + 31) / 32, grid = jit_grid(msg, n);
+  const int nw = (n + 31) / 32, grid = jit_grid(msg, n, defer);
   o << "#undef BCH_SV\n";
   if (scratch)
     o << "#define BCH_SV(u) scr[(u) * " << stride << "]\n";
@@ -444,12 +449,13 @@ static void emit_copy_body(std::ostringstream &o, const bch_code *c, int msg, in
 
 // The batch kernel's copy functor `name` (columns of stride `stride`).
 static void emit_copy(std::ostringstream &o, const bch_code *c, int msg, const std::string &name, int stride,
-                      bool scratch) {
-  o << "struct " << name << " {\n  static constexpr int kScratch = " << (scratch ? c->alg.n : 0) << ";\n"
+                      bool scratch, bool defer = false) {
+  o << "struct " << name << " {\n  static constexpr int kScratch = " << (scratch ? c->alg.n : 0)
+    << ";\n  static constexpr bool kDefer = " << (defer ? "true" : "false") << ";\n"
     << "  __device__ __forceinline__ void operator()(const SmemTables &, int, uint32_t, uint32_t,\n"
     << "      StoreT<" << msg << ">::Y *y, StoreT<" << msg << ">::A *acc, StoreT<" << msg
     << ">::A *scr, uint32_t jr, uint32_t sp, uint32_t, float alpha) const {\n";
-  emit_copy_body(o, c, msg, stride, scratch);
+  emit_copy_body(o, c, msg, stride, scratch, defer);
   o << "  }\n};\n";
 }
 
@@ -629,14 +635,14 @@ std::string jit_serve_blocks_source(const bch_code *const *codes, int n_codes) {
   return o.str();
 }
 
-static std::string jit_body_source(const bch_code *c, int msg) {
+static std::string jit_body_source(const bch_code *c, int msg, bool defer) {
   if (jit_split(c->alg.n)) return jit_split_source(c, msg);
   const int n = c->alg.n;
   const int tpb = jit_block_size(n);
   const int nw = (n + 31) / 32;
   std::ostringstream o;
   emit_prologue(o, msg, false);
-  emit_copy(o, c, msg, "JitCopy", tpb, jit_scratch_words(n) > 0);
+  emit_copy(o, c, msg, "JitCopy", tpb, jit_scratch_words(n) > 0, defer);
   o << "}  // namespace bchlib\n";
   o << "extern \"C\" __global__ void __launch_bounds__(" << tpb << ", " << jit_min_blocks(n)
     << ") bch_nms_jit(const bchlib::NmsArgs a) {\n"
@@ -945,7 +951,7 @@ static void write_file_atomic(const std::string &path, const std::vector<char> &
 
 // Returns the specialised kernel for (code, msg), compiling it on first use (or
 // loading it from the on-disk cache); on failure returns nullptr and sets *err.
-cudaKernel_t jit_kernel_from_source(const bch_code *c, int msg, std::string *err, int qfrac);
+cudaKernel_t jit_kernel_from_source(const bch_code *c, int msg, std::string *err, int qfrac, bool defer);
 
 // The tuning knobs that shape the generated source (read from the environment).
 static std::string jit_knob_signature(int n) {
@@ -960,14 +966,15 @@ static std::string jit_knob_signature(int n) {
 
 // The batch kernel's source for code c, format msg and qfrac fractional c2v bits (a
 // compile-time constant, so the other forms carry none of its branches).
-std::string jit_source(const bch_code *c, int msg, int qfrac) {
+std::string jit_source(const bch_code *c, int msg, int qfrac, bool defer) {
   return "#define BCH_JIT_QFRAC " + std::to_string(qfrac) + "\n" +
          (jit_copy_barrier() ? std::string() : std::string("#define BCH_JIT_NO_COPY_BARRIER 1\n")) +
-         jit_body_source(c, msg);
+         jit_body_source(c, msg, defer);
 }
 
-cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac) {
-  const std::string key = std::to_string(msg) + "/" + std::to_string(qfrac) + ":" + jit_knob_signature(c->alg.n);
+cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac, bool may_defer) {
+  const bool defer = may_defer && jit_defers(c->alg.n, msg);
+  const std::string key = std::string(defer ? "d" : "") + std::to_string(msg) + "/" + std::to_string(qfrac) + ":" + jit_knob_signature(c->alg.n);
   {
     std::lock_guard<std::mutex> lk(c->jit_mu);
     for (const auto &m : c->jit_memo)
@@ -977,7 +984,7 @@ cudaKernel_t jit_kernel(const bch_code *c, int msg, std::string *err, int qfrac)
       }
   }
   std::string why;
-  cudaKernel_t k = jit_kernel_from_source(c, msg, &why, qfrac);
+  cudaKernel_t k = jit_kernel_from_source(c, msg, &why, qfrac, defer);
   {
     std::lock_guard<std::mutex> lk(c->jit_mu);
     c->jit_memo.push_back({key, static_cast<void *>(k), why});
@@ -1064,8 +1071,8 @@ static cudaKernel_t compile_source(const std::string &src_in, const char *entry,
   return cp->kernel;
 }
 
-cudaKernel_t jit_kernel_from_source(const bch_code *c, int msg, std::string *err, int qfrac) {
-  return compile_source(jit_source(c, msg, qfrac), "bch_nms_jit", err);
+cudaKernel_t jit_kernel_from_source(const bch_code *c, int msg, std::string *err, int qfrac, bool defer) {
+  return compile_source(jit_source(c, msg, qfrac, defer), "bch_nms_jit", err);
 }
 
 // The row/column kernel of code c with FB slots per block for P copies;
@@ -1169,7 +1176,7 @@ bool jit_compile_check(const bch_code *c, int msg, std::string *log) {
     }
     rc_log += one;
   }
-  const bool ok = compile_check_source(jit_source(c, msg, 0), "bch_nms_jit", log);
+  const bool ok = compile_check_source(jit_source(c, msg, 0, jit_defers(c->alg.n, msg)), "bch_nms_jit", log);
   *log += rc_log;
   return ok;
 }

@@ -61,6 +61,13 @@ __device__ __forceinline__ uint32_t addmod(uint32_t a, uint32_t b, uint32_t n) {
   return __viaddmin_u32(x, 0u - n, x);
 }
 
+// max(a, b), NaN when one of them is.
+__device__ __forceinline__ float fmax_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 __device__ __forceinline__ float flip_sign(float mag, uint32_t sign_src) {
   return __uint_as_float(__float_as_uint(mag) ^ (sign_src & kSign));
 }
@@ -499,6 +506,11 @@ __device__ __forceinline__ int pull_frame(unsigned *queue, bool need, int F) {
 // straight-line copy code this keeps the instruction cache warm.
 template <int MSG, int NW, bool LOCKSTEP, int TPBC, class Copy>
 __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *smem, const Copy &copy) {
+  // kDefer (FP32): the copy takes a row's minima in a grid, which needs values without NaN.
+  // A frame that shows an infinity or NaN, in its input or after a merge, is put on the
+  // defer list, to be decoded from its input by the row/column kernel.
+  constexpr bool kDefer = MSG == kFP32 && Copy::kDefer;
+  static_assert(LOCKSTEP || !kDefer, "a lane whose frame is deferred stays in the block's loop");
   using Y = typename StoreT<MSG>::Y;
   using A = typename StoreT<MSG>::A;
   const int TPB = TPBC ? TPBC : int(blockDim.x);
@@ -533,6 +545,7 @@ __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *
         t = 0;
         escale = 0;
         const float *src = a.llr + size_t(f) * a.ld;
+        [[maybe_unused]] bool odd = false;
         float s4 = 4.0f;  // INT8 input scale: 4 (LSB 1/4), times 2^-k0 (see int8_input_shift)
         if constexpr (MSG == kINT8)
           if (BCH_QFRAC(a) && a.rescale) {
@@ -555,6 +568,7 @@ __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *
             if (i + h < n) {
               const float x = vv[h] + 0.0f;  // -0 -> +0: sgn(0) = +1
               if constexpr (MSG == kFP32) y[(i + h) * kShift] = x;
+              if constexpr (kDefer) odd |= !(fabsf(x) <= FLT_MAX);
               if constexpr (MSG == kFP16) y[(i + h) * kShift] = to_half_sat(x);
               if constexpr (MSG == kINT8) y[(i + h) * kShift] = to_q(s4 * x);
               acc[(i + h) * kShift] = A(0);
@@ -570,10 +584,17 @@ __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *
           const uint32_t sp = rs ? uint32_t(n) - rs : 0u;
           ctx[p * kShift] = j | (sp << 8);
         }
+        if constexpr (kDefer)
+          if (odd) {
+            a.defer[atomicAdd(a.defer_count, 1u)] = uint32_t(f);
+            f = -1;
+            need = true;
+          }
       }
     }
     if constexpr (LOCKSTEP) {
-      if (!__syncthreads_or(f >= 0)) break;
+      // (a slot whose frame was deferred runs idle this iteration and pulls its next one)
+      if (!__syncthreads_or(f >= 0 || (kDefer && need))) break;
     } else {
       if (!__any_sync(kFull, f >= 0)) break;
       if (f < 0) continue;
@@ -600,9 +621,15 @@ __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *
           y[i * kShift] = yn;
           acc[i * kShift] = 0.0f;
           cb[i >> 5] |= (__float_as_uint(yn) >> 31) << (i & 31);
-          mx = fmaxf(mx, fabsf(yn));
+          mx = kDefer ? fmax_nan(mx, fabsf(yn)) : fmaxf(mx, fabsf(yn));
         }
       }
+      if constexpr (kDefer)
+        if (f >= 0 && !(mx <= FLT_MAX)) {
+          a.defer[atomicAdd(a.defer_count, 1u)] = uint32_t(f);
+          f = -1;
+          need = true;
+        }
       // y grows about tenfold per iteration; past 2^100 the frame is scaled by 2^-64
       // (exact, and min-sum is scale invariant) so that long decodes of high-degree
       // codes cannot overflow FP32.  Not in training, whose checkpoints are in LLR units.
@@ -900,6 +927,7 @@ __device__ __forceinline__ void nms_split_persistent(const NmsArgs &a, unsigned 
 template <int MSG, int WB>
 struct GenericCopy {
   static constexpr int kScratch = 0;
+  static constexpr bool kDefer = false;
   __device__ __forceinline__ void operator()(const SmemTables &tb, int n_groups, uint32_t n, uint32_t m,
                                              typename StoreT<MSG>::Y *y, typename StoreT<MSG>::A *acc,
                                              typename StoreT<MSG>::A *, uint32_t jr, uint32_t sp,

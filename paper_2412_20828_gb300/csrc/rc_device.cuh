@@ -427,6 +427,10 @@ template <int MSG>
 __device__ __forceinline__ void rc_persistent(const NmsArgs &a, uint32_t *sm) {
   using V = typename RcV<MSG>::T;
   constexpr int FB = RC_FB, YS = FB == 32 ? 33 : FB, NW = (RC_N + 31) / 32, KW = RC_KW;
+  // the frames of this launch: 0 .. F - 1, or those of a list another kernel wrote
+  const int n_frames = a.list ? int(min(*a.list_count, unsigned(a.F))) : a.F;
+  if (int(blockIdx.x) * FB >= n_frames) return;
+  auto frame = [&](int i) { return i < 0 || i >= n_frames ? -1 : a.list ? int(a.list[i]) : i; };
   const int P = RC_PC ? RC_PC : a.P, tid = int(threadIdx.x), nthr = int(blockDim.x);
   // the shuffle tells the compiler that the warp index, and with it every table index
   // computed from it, is uniform
@@ -479,8 +483,7 @@ __device__ __forceinline__ void rc_persistent(const NmsArgs &a, uint32_t *sm) {
   // Lane s of every warp holds slot s's frame, iteration count and exponent.  The block's
   // first frames are fixed; later ones come from the queue.
   const int start = int(gridDim.x) * FB;
-  int my_f = lane < FB ? int(blockIdx.x) * FB + lane : -1, my_t = 0, my_e = 0;
-  if (my_f >= a.F) my_f = -1;
+  int my_f = lane < FB ? frame(int(blockIdx.x) * FB + lane) : -1, my_t = 0, my_e = 0;
   uint32_t nw = __ballot_sync(kFull, my_f >= 0);
   for (;;) {
     if (nw) {
@@ -654,10 +657,10 @@ __device__ __forceinline__ void rc_persistent(const NmsArgs &a, uint32_t *sm) {
         for (int i = lane; i < RC_N; i += 32) dst[i] = ldexpf(float(y_s[i * YS + s]) * unit, e);
       }
     }
-    if (a.F > start) {
+    if (n_frames > start) {
       if (warp == 0) {
-        const int got = pull_frame(a.queue, fin, a.F - start);
-        if (fin) f_s[lane] = got >= 0 ? got + start : -1;
+        const int got = pull_frame(a.queue, fin, n_frames - start);
+        if (fin) f_s[lane] = got >= 0 ? frame(got + start) : -1;
       }
       __syncthreads();
       if (fin) my_f = f_s[lane];
