@@ -733,8 +733,10 @@ static bool rc_fits(const bch_code *code, const NmsArgs &a, int FB) {
 //    349, 16 384 frames 300+ / 182 / 350; BCH(127,64), ep 8670, 1531 frames 138 / 218 / 1322,
 //    4096 frames 310 / 219 / 1322; BCH(63,36) with 9 copies 2400 frames 90 / 109 / 321, 4800
 //    frames 163 / 110 / 322;
-//  * n <= 63, three copies: 32 slots up to 160 (FP16 300, INT8 176) frames per SM, the crossing
-//    where every frame is hard (1 to 2 dB: 20 000 frames - / 306 / 351, 30 000 - / 424 / 354);
+//  * n <= 63, three copies: 32 slots up to 136 (FP16 224, INT8 152) frames per SM, the crossing
+//    where every frame is hard (BCH(63,36), 1 to 2 dB, 32 slots / one thread: FP32 128 per SM 302 /
+//    329, 144 per SM 341 / 328; FP16 200 per SM 522 / 568, 256 per SM 631 / 566; INT8 144 per SM
+//    493 / 530, 160 per SM 552 / 531; over 1 to 6 dB 32 slots win by 1.4 to 1.9 there);
 //    other numbers of copies, whose loops are not unrolled, up to 64;
 //  * beyond ~1000 edges the straight-line rows outgrow the instruction cache and 32 slots win
 //    at any size: BCH(127,64) 100 000 frames - / 2731 / 5384, BCH(127,99) - / 2156 / 4232,
@@ -751,7 +753,7 @@ static int rc_slots(const bch_code *code, const NmsArgs &a, int sms) {
   const int ep = std::max(1, code->dc.edges * a.P), one = fits32 || cached ? std::min(64, 8 + 61200 / ep) : 112;
   if (a.F <= sms * one && rc_fits(code, a, 1)) return 1;
   if (!fits32) return 0;
-  const int many = a.P != 3 ? 64 : a.msg == BCH_MSG_FP16 ? 300 : a.msg == BCH_MSG_INT8 ? 176 : 160;
+  const int many = a.P != 3 ? 64 : a.msg == BCH_MSG_FP16 ? 224 : a.msg == BCH_MSG_INT8 ? 152 : 136;
   return !cached || a.F <= sms * many ? 32 : 0;
 }
 
