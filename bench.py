@@ -308,7 +308,8 @@ def nms_roofline(B, torch, dev, clocks, edge_updates, nms_time, kinfo, frames, n
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_lane_ops / 1e12,
             "unit": "Tlane-op/s", "frac": achieved / peak_lane_ops, "traffic": traffic,
             "traffic_unit": "bytes per launch", "algorithmic_bytes_per_launch": frames * (n * 4 + W64 * 8 + 2),
-            "kernel": "bch_nms_jit" if kinfo == "jit" else "nms_enhanced_kernel", "kernel_info": kinfo,
+            "kernel": ("bch_nms_jit" if n <= 63 else "bch_nms_rc") if kinfo == "jit" else "nms_enhanced_kernel",
+            "kernel_info": kinfo,
             "lane_ops_per_edge_update": LANE_OPS_PER_EDGE, "edge_updates_per_s": edge_updates / nms_time,
             "nms_ms_per_step": nms_time * 1e3,
             "peak_basis": f"{sms} SMs x 128 lanes x {clk_mhz:.0f} MHz (median SM clock under load)",
