@@ -46,8 +46,8 @@ struct NmsArgs {
   float *ckpt;  // training checkpoints [I+1][F][ld] or null
   unsigned *queue;
   unsigned *check;  // checked builds: the device's check word [4]; else unused
-  // frames the straight-line FP32 kernel leaves to the row/column kernel (an infinity or NaN
-  // among their values), and that kernel's list of frames (null: frames 0 .. F - 1)
+  // frames the straight-line FP32 kernel leaves to the row/column kernel (a NaN among their
+  // values), and that kernel's list of frames (null: frames 0 .. F - 1)
   uint32_t *defer;
   unsigned *defer_count;
   const uint32_t *list;

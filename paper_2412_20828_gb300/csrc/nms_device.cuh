@@ -507,8 +507,9 @@ __device__ __forceinline__ int pull_frame(unsigned *queue, bool need, int F) {
 template <int MSG, int NW, bool LOCKSTEP, int TPBC, class Copy>
 __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *smem, const Copy &copy) {
   // kDefer (FP32): the copy takes a row's minima in a grid, which needs values without NaN.
-  // A frame that shows an infinity or NaN, in its input or after a merge, is put on the
-  // defer list, to be decoded from its input by the row/column kernel.
+  // A frame that shows a NaN, in its input or after a merge, is put on the defer list, to be
+  // decoded from its input by the row/column kernel.  Infinite LLRs (known or erased bits)
+  // stay here: 10^6 frames of BCH(63,36) with nine of them each take 3.5 ms, deferred 23.7 ms.
   constexpr bool kDefer = MSG == kFP32 && Copy::kDefer;
   static_assert(LOCKSTEP || !kDefer, "a lane whose frame is deferred stays in the block's loop");
   using Y = typename StoreT<MSG>::Y;
@@ -568,7 +569,7 @@ __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *
             if (i + h < n) {
               const float x = vv[h] + 0.0f;  // -0 -> +0: sgn(0) = +1
               if constexpr (MSG == kFP32) y[(i + h) * kShift] = x;
-              if constexpr (kDefer) odd |= !(fabsf(x) <= FLT_MAX);
+              if constexpr (kDefer) odd |= x != x;
               if constexpr (MSG == kFP16) y[(i + h) * kShift] = to_half_sat(x);
               if constexpr (MSG == kINT8) y[(i + h) * kShift] = to_q(s4 * x);
               acc[(i + h) * kShift] = A(0);
@@ -625,7 +626,7 @@ __device__ __forceinline__ void nms_persistent(const NmsArgs &a, unsigned char *
         }
       }
       if constexpr (kDefer)
-        if (f >= 0 && !(mx <= FLT_MAX)) {
+        if (f >= 0 && mx != mx) {
           a.defer[atomicAdd(a.defer_count, 1u)] = uint32_t(f);
           f = -1;
           need = true;

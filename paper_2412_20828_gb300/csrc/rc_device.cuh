@@ -53,7 +53,7 @@ struct RcPtr {
   const uint2 *rows, *cols;
   int P, task, stride;
   float alpha;
-  bool slow;  // the warp holds a frame with an infinity or NaN
+  bool slow;  // the warp holds a frame with a NaN
 };
 
 template <int MSG>
@@ -62,7 +62,7 @@ __device__ __forceinline__ typename RcV<MSG>::T rc_ld(const unsigned char *p) {
 }
 
 // ---------------------------------------------------------------- rows
-// min1 / min2 of a row with infinities or NaN among its values, in the order of the
+// min1 / min2 of a row with a NaN among its values, in the order of the
 // one-thread-per-frame kernels (fminf / fmaxf pass over a NaN, and a NaN edge lowers min2
 // to the running min1; n = 127: two halves of the variables, then joined).  off(e): byte
 // offset of edge e's value.
@@ -178,7 +178,9 @@ __device__ __forceinline__ void rc_rows(const RcPtr &c, int nr, int r0, int t0) 
 #pragma unroll
       for (int e = 0; e < W; e++) sg ^= rc_take(v[e]);
       min12<V, W>(v, m1, m2);
-      if constexpr (MSG == kFP32)
+      if constexpr (MSG == kFP32) {
+        m1 = fminf(m1, FLT_MAX);  // the running pair's start value, which rows of infinities show
+        m2 = fminf(m2, FLT_MAX);
         if (c.slow) {
           const float2 o = rc_min12_ordered(c.z + p * (kRcZP * 128), W, [&](int e) {
             return reinterpret_cast<const int *>(rc_rowtab)[4 * t0 + t * ((W + 3) & ~3) + e];
@@ -186,6 +188,7 @@ __device__ __forceinline__ void rc_rows(const RcPtr &c, int nr, int r0, int t0) 
           m1 = o.x;
           m2 = o.y;
         }
+      }
       rc_store_row<MSG>(c, (p * kRcRP + r0 + t) * 32, m1, m2, sg);
     }
   }
@@ -502,7 +505,7 @@ __device__ __forceinline__ void rc_persistent(const NmsArgs &a, uint32_t *sm) {
         if constexpr (MSG == kFP32) {
           bool odd = false;
 #pragma unroll
-          for (int w = 0; w < NW; w++) odd |= !(fabsf(x[w]) <= FLT_MAX);
+          for (int w = 0; w < NW; w++) odd |= x[w] != x[w];
           const bool any = __any_sync(kFull, odd);
           if (lane == 0) bad_s[s] = any ? 1u : 0u;
         }
@@ -571,12 +574,11 @@ __device__ __forceinline__ void rc_persistent(const NmsArgs &a, uint32_t *sm) {
       }
       if constexpr (MSG == kFP32) {
         if (__any_sync(kFull, live && m.large)) {
-          // rare: mark the slots with a finite or infinite value past 2^100, and those with
-          // an infinity or NaN
+          // rare: mark the slots with a finite or infinite value past 2^100, and those with a NaN
           for (int i = i0; i < i1; i++) {
             const float v = fabsf(y[i * YS]);
             if (v > 0x1p100f) mx_s[slot] = 1u;
-            if (!(v <= FLT_MAX)) bad_s[slot] = 1u;
+            if (v != v) bad_s[slot] = 1u;
           }
         }
       } else if (a.rescale) {
