@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -726,35 +727,64 @@ static bool rc_fits(const bch_code *code, const NmsArgs &a, int FB) {
 
 // The row/column kernel (frame slots per block: 1 or 32) for this call, or 0 when the
 // one-thread-per-frame kernel is the better one.  BCHDEC_JIT_RC=0|1|32 overrides (a tuning
-// and comparison knob; all compute the same bits).  The lines lie where the measured times
-// cross (GB300, 12 iterations, Eb/N0 U[1, 6) dB unless said; us for 1 slot / 32 slots / one
-// thread per frame; ep = edges x copies of one iteration):
-//  * one slot up to 8 + 61200 / ep frames per SM: BCH(63,36), ep 2550, 4096 frames 77 / 91 /
-//    349, 16 384 frames 300+ / 182 / 350; BCH(127,64), ep 8670, 1531 frames 138 / 218 / 1322,
-//    4096 frames 310 / 219 / 1322; BCH(63,36) with 9 copies 2400 frames 90 / 109 / 321, 4800
-//    frames 163 / 110 / 322;
-//  * n <= 63, three copies: 32 slots up to 136 (FP16 224, INT8 152) frames per SM, the crossing
-//    where every frame is hard (BCH(63,36), 1 to 2 dB, 32 slots / one thread: FP32 128 per SM 302 /
-//    329, 144 per SM 341 / 328; FP16 200 per SM 522 / 568, 256 per SM 631 / 566; INT8 144 per SM
-//    493 / 530, 160 per SM 552 / 531; over 1 to 6 dB 32 slots win by 1.4 to 1.9 there);
-//    other numbers of copies, whose loops are not unrolled, up to 64;
-//  * beyond ~1000 edges the straight-line rows outgrow the instruction cache and 32 slots win
-//    at any size: BCH(127,64) 100 000 frames - / 2731 / 5384, BCH(127,99) - / 2156 / 4232,
-//    BCH(63,36) with 122 rows 200 000 frames - / 2032 / 2827;
-//  * where the copies of 32 frames exceed shared memory (n = 127, five copies or more) one
-//    slot wins up to about 112 frames per SM: nine copies 10 000 frames 822 / - / 1318, 25 000
-//    frames 2011 / - / 2000.
+// and comparison knob; all compute the same bits).  The lines, in frames per SM, lie where no
+// call is slower than on the one-thread-per-frame kernel, also when every frame runs all its
+// iterations (no early stop, or 1 to 2 dB).  Easy frames gain past a line too, but the host
+// cannot know them.  us on a GB300 for 1 slot / 32 slots / one thread per frame, 12 iterations
+// unless said; ep = edges x copies:
+//  * one slot: a frame's iteration costs an SM 0.21 us per 1000 ep, at least 0.18 us.  Up to 8 +
+//    61200 / ep frames, where 32 slots win at 1 to 6 dB (BCH(63,36) 4096 frames 77 / 91 / 349, 16 384
+//    frames 300+ / 182 / 350; BCH(127,64) 1531 frames 138 / 218 / 1322, 4096 frames 310 / 219 / 1322), and up to
+//    40 (no early stop: BCH(63,45), two copies, 8 iterations 61 per SM 159 / - / 137; BCH(63,57) 45 per SM
+//    201 / - / 193); n = 15 up to 4 (nine copies, no early stop, 63 per SM 323 / 75 / 115);
+//  * n <= 63, three copies, 32 slots (64 frames of an SM at a time): with 8 iterations or more and
+//    early stop up to 136 per SM, FP16 224, INT8 152 (BCH(63,36) at 1 to 2 dB: FP32 136 per SM - / 322 /
+//    353, 144 per SM - / 341 / 328; FP16 224 per SM - / 571 / 625; INT8 152 per SM - / 543 / 634).  Without
+//    early stop, or with few iterations, where refilling the slots shows, up to 96, FP16 160,
+//    INT8 128 (FP32 BCH(63,36) 96 per SM, 4 iterations at 1 to 2 dB - / 107 / 129, 128 per SM - / 142 / 129;
+//    BCH(63,57) 128 per SM, no early stop, - / 217 / 194; FP16 BCH(63,45) 160 per SM - / 350 / 384, 192 per SM
+//    - / 410 / 386; INT8 BCH(63,36) 152 per SM - / 650 / 631); n = 15 then up to 64;
+//  * other numbers of copies, whose loops are not unrolled, up to 64: BCH(63,36), no early stop, 64
+//    per SM one copy 147 / 117 / 149, nine copies 1518 / 607 / 940;
+//  * n = 63 beyond ~1000 edges the straight-line rows outgrow the instruction cache: BCH(63,36)
+//    with 122 rows, no early stop, three copies 1000 per SM - / 4788 / 5346 (FP32, FP16: any size);
+//    INT8 300 per SM - / 2250 / 3069, 1000 per SM - / 7164 / 6253; one copy 64 per SM - / 250 / 489, 128 per SM at
+//    1 to 2 dB - / 530 / 494 (FP16 - / 480 / 651); two copies 200 per SM - / 1147 / 920;
+//  * n = 127: 32 slots at any size: BCH(127,64) 100 000 frames - / 2731 / 5384, BCH(127,99) - / 2156 /
+//    4232, FP16 and INT8 BCH(127,64) 300 per SM - / 1522 / 4032 and - / 1920 / 4116, four copies BCH(127,99) - /
+//    1992 / 3261.  With one or two copies the other kernel's single round of 128 frames per SM is
+//    quicker: one copy 100 per SM BCH(127,64) - / 575 / 544, BCH(127,99) - / 567 / 411, and for ep < 2800
+//    later rounds too (BCH(127,78) 500 per SM, no early stop, - / 2305 / 2120);
+//  * where the copies of 32 frames exceed shared memory (four or five copies or more), one slot
+//    up to the crossing where every frame runs on: n = 127, nine copies, 4 iterations, 80 per SM
+//    BCH(127,64) 1439 / - / 1400, BCH(127,99) 1220 / - / 1052, INT8 1612 / - / 1203; one iteration, five copies
+//    60 per SM 231 / - / 205; BCH(63,36) with 122 rows, nine copies 64 per SM 2528 / - / 3896, INT8, four
+//    copies, 80 per SM 2275 / - / 2076.
 static int rc_slots(const bch_code *code, const NmsArgs &a, int sms) {
   if (const char *v = std::getenv("BCHDEC_JIT_RC")) {
     const int fb = std::atoi(v);
     return (fb == 1 || fb == 32) && rc_fits(code, a, fb) ? fb : 0;
   }
-  const bool fits32 = rc_fits(code, a, 32), cached = code->alg.n <= 63 && code->dc.edges <= 1000;
-  const int ep = std::max(1, code->dc.edges * a.P), one = fits32 || cached ? std::min(64, 8 + 61200 / ep) : 112;
-  if (a.F <= sms * one && rc_fits(code, a, 1)) return 1;
+  const int n = code->alg.n, ep = std::max(1, code->dc.edges * a.P);
+  const bool fits32 = rc_fits(code, a, 32), cached = n <= 63 && code->dc.edges <= 1000;
+  auto within = [&](int per_sm) { return a.F <= (long long)sms * per_sm; };
+  auto by_format = [&](int fp32, int fp16, int int8) {
+    return a.msg == BCH_MSG_FP16 ? fp16 : a.msg == BCH_MSG_INT8 ? int8 : fp32;
+  };
+  int one = 0;
+  if (n < 63) one = 4;
+  else if (fits32 || cached) one = std::min(40, 8 + 61200 / ep);
+  else if (n == 63) one = by_format(80, 80, 64);
+  else one = a.I < 4 ? 48 : by_format(60, 64, 50);
+  if (within(one) && rc_fits(code, a, 1)) return 1;
   if (!fits32) return 0;
-  const int many = a.P != 3 ? 64 : a.msg == BCH_MSG_FP16 ? 224 : a.msg == BCH_MSG_INT8 ? 152 : 136;
-  return !cached || a.F <= sms * many ? 32 : 0;
+  if (n > 63) return a.P < 3 && !within(64) && (within(128) || ep < 2800) ? 0 : 32;
+  int many = 64;
+  if (a.P == 3 && !cached) many = by_format(INT_MAX, INT_MAX, 300);
+  else if (a.P == 3 && a.I >= 8 && a.early_stop) many = by_format(136, 224, 152);
+  else if (a.P == 3 && n == 63) many = by_format(96, 160, 128);
+  else if (!cached && (a.P == 2 || (a.P == 1 && a.msg != BCH_MSG_FP32))) many = 128;
+  return within(many) ? 32 : 0;
 }
 
 static cudaError_t launch_rc(cudaKernel_t k, int FB, const bch_code *code, const NmsArgs &a, cudaStream_t st,
@@ -800,6 +830,9 @@ static int rcp_slots(const bch_code *code, const NmsArgs &a, int sms) {
     const int fb = std::atoi(v);
     return (fb == 1 || fb == 16 || fb == 32) && fits(fb) ? fb : 0;
   }
+  // n = 15: a frame is so short a chain that large batches run better one thread each: BCH(15,7)
+  // 10 000 frames 23 / 47 (32 slots / precompiled), 300 000 frames 203 / 120
+  if (code->alg.n < 63 && a.F > sms * 64LL) return 0;
   if (a.F <= sms * 8 && fits(1)) return 1;
   if (a.F <= sms * 16 && fits(16)) return 16;
   return fits(32) ? 32 : fits(16) ? 16 : fits(1) ? 1 : 0;
@@ -838,8 +871,9 @@ static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaS
     if (fb)
       if (cudaKernel_t k = jit_rcp_kernel(code, fb, &err)) return launch_rcp(k, fb, code, a, st, cleared);
   }
+  int sms = 0;
   if (a.P > 0 && mode != 1) {
-    int dev = 0, sms = 0;
+    int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
@@ -860,7 +894,10 @@ static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaS
     // frames of BCH(63,36) with a NaN in each 22 ms, with one slot 42 ms
     cudaKernel_t rk = nullptr;
     const int rfb = rc_fits(code, a, 32) ? 32 : 1;
-    if (jit_defers(code->alg.n, a.msg) && rc_fits(code, a, rfb))
+    // (a call of little work keeps the edge order and spares the second launch, 3 to 7 us: one
+    // iteration of 60 800 frames of BCH(63,36), one copy, 42.8 / 49.6 us, three copies 74.8 / 78.3 us)
+    const long long work = (long long)a.F * a.I * code->dc.edges * a.P;
+    if (work >= 2000000LL * sms && jit_defers(code->alg.n, a.msg) && rc_fits(code, a, rfb))
       rk = jit_rc_kernel(code, a.msg, a.qfrac, rfb, a.P, &err);
     cudaKernel_t k = jit_kernel(code, a.msg, &err, a.qfrac, rk != nullptr);
     if (k) {

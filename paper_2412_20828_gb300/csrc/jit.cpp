@@ -333,10 +333,12 @@ static void emit_chain_loop(std::ostringstream &o, int n, const std::string &stm
 // FP32 (0 / 1 / 2): (63,36) 3353 / 3119 / 3239, (63,45) 1837 / 1752 / 1746; a NaN is passed over by
 // its position in the edge order, so the batch kernel then defers frames with one (defer;
 // the serving kernels, which cannot, keep the edge order).  Infinities need only the edge
-// order's start value FLT_MAX on both minima (0.2% of 3 000 000 frames of BCH(63,36)).
+// order's start value FLT_MAX on both minima (0.2% of 3 000 000 frames of BCH(63,36)).  n = 15 keeps the
+// edge order in FP32: the second launch costs its calls more (20 672 frames of BCH(15,7), one
+// copy, 28 / 33 us).
 static int jit_grid(int msg, int n, bool defer) {
   if (n > 63 || !jit_incr() || env_int("BCHDEC_JIT_GRID", 0, 1, 1) == 0) return 0;
-  return msg == 1 ? 1 : msg == 2 ? 2 : defer ? 1 : 0;
+  return msg == 1 ? 1 : msg == 2 ? 2 : defer && n == 63 ? 1 : 0;
 }
 // Whether the batch kernel of format msg defers frames (see jit_grid).
 bool jit_defers(int n, int msg) { return msg == 0 && jit_grid(0, n, true) != 0; }
