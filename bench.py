@@ -292,7 +292,7 @@ def run_plain(B, torch, dev, reps=50):
             "edge_updates_per_s": float(c[5]) * 486 / dt}
 
 
-def nms_roofline(B, torch, dev, clocks, edge_updates, nms_time, kinfo, frames, n, traffic_per_frame):
+def nms_roofline(torch, dev, clocks, edge_updates, nms_time, kernel, frames, n, traffic_per_frame):
     """Roofline of the enhanced-NMS kernel: ALU lane-ops (8 per edge update) per second
     against SMs x 128 lanes x the median SM clock under load."""
     peaks = measured_peaks()
@@ -301,15 +301,14 @@ def nms_roofline(B, torch, dev, clocks, edge_updates, nms_time, kinfo, frames, n
     peak_lane_ops = sms * 128 * clk_mhz * 1e6
     achieved = edge_updates * LANE_OPS_PER_EDGE / nms_time
     traffic = None
-    if kinfo == "jit" and traffic_per_frame is not None:
+    if kernel.startswith("bch_") and traffic_per_frame is not None:
         traffic = traffic_per_frame * frames  # bytes per launch (one code's frames)
     W64 = (n + 63) // 64
     ld = 64 if n <= 63 else 128
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_lane_ops / 1e12,
             "unit": "Tlane-op/s", "frac": achieved / peak_lane_ops, "traffic": traffic,
             "traffic_unit": "bytes per launch", "algorithmic_bytes_per_launch": frames * (n * 4 + W64 * 8 + 2),
-            "kernel": ("bch_nms_jit" if n <= 63 else "bch_nms_rc") if kinfo == "jit" else "nms_enhanced_kernel",
-            "kernel_info": kinfo,
+            "kernel": kernel,
             "lane_ops_per_edge_update": LANE_OPS_PER_EDGE, "edge_updates_per_s": edge_updates / nms_time,
             "nms_ms_per_step": nms_time * 1e3,
             "peak_basis": f"{sms} SMs x 128 lanes x {clk_mhz:.0f} MHz (median SM clock under load)",
@@ -384,7 +383,7 @@ def run_config4(B, torch, dev, clocks, frames_per_point, steps=2, warmup=1):
         nms_t = sum(a.elapsed_time(b) for a, b in st["ev"]) / 1e3 / steps
         ctr = st["ctr"].cpu().numpy()
         eu = int(ctr[:, 5].sum()) * P_AUTOS * st["code"].edges
-        kinfo = st["code"].kernel_info(B.MSG_FP32, P_AUTOS)
+        kernel = st["code"].kernel_name(st["p"], F)
         pts = []
         for pi, e in enumerate(CONFIG4_POINTS):
             c = ctr[pi]
@@ -392,7 +391,7 @@ def run_config4(B, torch, dev, clocks, frames_per_point, steps=2, warmup=1):
                         "ber": c[2] / (c[0] * st["n"]), "nms_fer": 1 - c[6] / c[0],
                         "avg_iters": c[5] / c[0], "osd_frames": int(c[4])})
         out["codes"][f"({st['n']},{st['k']})"] = {
-            "roofline": nms_roofline(B, torch, dev, clocks, eu, nms_t, kinfo, F, st["n"],
+            "roofline": nms_roofline(torch, dev, clocks, eu, nms_t, kernel, F, st["n"],
                                      JIT127_DRAM_BYTES_PER_FRAME if st["n"] == 127 else None),
             "per_point": pts}
         st["code"].close()
@@ -611,8 +610,8 @@ def main():
     ms = elapsed / args.steps * 1e3
     value = D.job_throughput(frames_per_step, world, elapsed / args.steps)
     eups = edge_updates / nms_time
-    kinfo = states[0]["code"].kernel_info(msg, P_AUTOS)
-    roofline = nms_roofline(B, torch, dev, clocks, edge_updates, nms_time, kinfo, F, 63,
+    kernel = states[0]["code"].kernel_name(states[0]["p"], F)
+    roofline = nms_roofline(torch, dev, clocks, edge_updates, nms_time, kernel, F, 63,
                             JIT_DRAM_BYTES_PER_FRAME if msg == B.MSG_FP32 else None)
 
     # the step's decisions on the oracle's sample (frames 0..N-1 of every point), taken
@@ -630,7 +629,6 @@ def main():
     legs = {"fp32": dict(msg=B.MSG_FP32), "fp16": dict(msg=B.MSG_FP16), "int8": dict(msg=B.MSG_INT8),
             "int8f": dict(msg=B.MSG_INT8, rescale=True, qfrac=8)}
     for name in [x for x in args.msg_legs.split(",") if x and x != args.msg]:
-        mv = legs[name]["msg"]
         saved = [st["p"] for st in states]
         for st in states:
             st["p"] = B.params(ITERS, ALPHA, n_autos=P_AUTOS, early_stop=True, osd_order=OSD_ORDER, **legs[name])
@@ -649,8 +647,8 @@ def main():
         eu = sum(int(st["iters"].long().sum()) * P_AUTOS * st["code"].edges for st in states)
         fe = [int((st["hard"] != st["cw"]).any(dim=1).sum()) for st in states]
         msg_legs[name] = {"frames_per_s": frames_per_step / t_leg, "ms_per_step": t_leg * 1e3,
-                          "roofline": nms_roofline(B, torch, dev, clocks, eu, nt,
-                                                   states[0]["code"].kernel_info(mv, P_AUTOS), F, 63, None),
+                          "roofline": nms_roofline(torch, dev, clocks, eu, nt,
+                                                   states[0]["code"].kernel_name(states[0]["p"], F), F, 63, None),
                           "frame_errors_per_code": fe}
         for st, p0 in zip(states, saved):
             st["p"] = p0

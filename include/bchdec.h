@@ -146,23 +146,41 @@ bch_status bch_build_pcm_host(int n, int k, bch_pcm_kind kind, int m_rows, uint6
                               const bch_pcm_opts *opts, uint8_t *dense, size_t capacity,
                               int *rows);
 
-/* Names the enhanced-NMS kernel a decode of `code` with storage `msg` and n_autos
- * automorphisms runs: "jit" -- the kernel compiled at run time (NVRTC) for this code's
- * Tanner graph, rows as straight-line code on registers -- or "generic: <reason>" --
- * the precompiled kernel that reads the rows from shared memory.  The environment
- * variable BCHDEC_NMS_KERNEL=generic|jit|auto selects (default auto: jit when it
- * compiles, else generic; for n = 127 the specialised kernel is about 1.8x faster than
- * the precompiled one).  The first call for a code compiles (a few seconds for n <= 63,
- * 30-90 s for n = 127) and caches the kernel in the process and on disk
- * (BCHDEC_JIT_CACHE_DIR, default $XDG_CACHE_HOME/bchdec or $HOME/.cache/bchdec; "off"
- * disables it).  Tuning knobs of the specialised kernel, read when its source is
- * generated: BCHDEC_JIT_TPB (block size for n <= 63), BCHDEC_JIT_MIN_BLOCKS (register
- * budget), BCHDEC_JIT_PAIRS (min1/min2 two edges at a time), BCHDEC_JIT_FMA_PCT (share
- * of edges whose min2 correction runs on the FMA pipe), BCHDEC_JIT_ROW_FENCE (compiler
- * fence between rows), BCHDEC_JIT_DUMP (file receiving the source, with
- * bch_nms_jit_check).  Every setting computes the same results. */
+/* Min-sum kernels.  A decode runs a kernel compiled at run time (NVRTC) for the code's
+ * Tanner graph; which one depends on the code, the format, the number of automorphisms
+ * and the number of frames: a row/column kernel with one frame per block (bch_nms_rc; the
+ * smallest calls) or 32 (middle sizes, and most sizes of n = 127), one thread per frame
+ * with the rows as straight-line code on registers (bch_nms_jit; large batches; the FP32
+ * one of n = 63 leaves frames with a NaN to bch_nms_rc), and bch_plain_rc for the plain
+ * decoder.  Precompiled kernels that read the rows from shared memory stand in where a
+ * kernel does not compile, and run the largest batches of the plain decoder at n = 15.
+ * The run-time kernels give a frame the same bits whichever of them decodes it.
+ * Each kernel compiles on first use (1 to 10 s, bch_nms_jit of n = 127 the longest) and is
+ * cached in the process and on disk (BCHDEC_JIT_CACHE_DIR, default $XDG_CACHE_HOME/bchdec or
+ * $HOME/.cache/bchdec; "off" disables it).  A first use may be under stream capture.
+ * Environment: BCHDEC_NMS_KERNEL=generic|jit|auto (default auto; generic: the precompiled
+ * kernels; jit: fail instead of falling back), BCHDEC_JIT_RC=0|1|16|32 (frames per block of the
+ * row/column kernels, 16 for the plain decoder only, 0 for none) and tuning knobs, read when a
+ * source is generated: BCHDEC_JIT_GRID=0 (min1/min2 of the straight-line rows in edge order),
+ * BCHDEC_JIT_TPB (block size for n <= 63), BCHDEC_JIT_MIN_BLOCKS (register budget),
+ * BCHDEC_JIT_PAIRS (min1/min2 two edges at a time), BCHDEC_JIT_FMA_PCT (share of edges whose
+ * min2 correction runs on the FMA pipe), BCHDEC_JIT_ROW_FENCE (compiler fence between rows),
+ * BCHDEC_JIT_DUMP (file receiving the source, with bch_nms_jit_check).  Every knob computes
+ * the same results.
+ *
+ * bch_nms_kernel_info compiles and loads the kernels that decodes of `code` with storage
+ * `msg` (qfrac = 0) and n_autos automorphisms run at any number of frames, so that no such
+ * decode compiles later, and writes "jit", or "generic: <reason>" when only the precompiled
+ * kernels are available ("jit; some sizes generic: <reason>" when some are not). */
 bch_status bch_nms_kernel_info(const bch_code *code, int msg, int n_autos, char *buf,
                                size_t capacity);
+
+/* Compiles and loads the min-sum kernels that bch_nms_decode of n_frames >= 1 frames with
+ * these parameters runs, and writes their names: "bch_nms_rc", "bch_nms_jit",
+ * "bch_nms_jit + bch_nms_rc" (the second over the deferred frames), "bch_plain_rc",
+ * "nms_enhanced_kernel" or "nms_plain_kernel" (precompiled).  Launches nothing. */
+bch_status bch_nms_kernel_name(const bch_code *code, const bch_nms_params *params, int n_frames,
+                               char *buf, size_t capacity);
 
 /* Compiles the run-time specialised enhanced-NMS kernel for the optimized matrix that
  * bch_build_pcm(n, k, BCH_PCM_OPTIMIZED, m_rows, seed, opts) builds, for sm_103a with
@@ -278,7 +296,7 @@ bch_status bch_hybrid_decode_noalloc(const bch_code *code, const bch_code *std_c
 /* Failed-frame compaction (the hybrid decoder's hand-off to OSD): writes to list
  * (device [n_frames] u32) the indices of the frames whose flags lack
  * BCH_FLAG_CONVERGED, in ascending order, and their number to *count (device u32).
- * Deterministic two-pass block scan; no host synchronisation. */
+ * Deterministic block scan (one launch up to 8192 frames, else two); no host synchronisation. */
 bch_status bch_compact_failed(const uint8_t *flags, int n_frames, uint32_t *list, uint32_t *count,
                               void *workspace, void *stream);
 
@@ -462,7 +480,9 @@ bch_status bch_nms_forward_train(const bch_code *code, const bch_nms_params *par
  * [n_frames][ld] (nullable) and grad_alpha[iters] (device FP32, overwritten).
  * d c2v/d alpha_t = c2v/alpha_t; d c2v(j,u)/d z_a = alpha_t prod_{u'!=u} sgn z_u' sgn z_a
  * at a = argmin over the row without u (lowest column on ties); sign derivatives 0.
- * Recomputes each iteration from its checkpoint. */
+ * Recomputes each iteration from its checkpoint.  Runs a kernel compiled at run time for the
+ * code (bch_bwd_rc; on first use, as the decoders' kernels), or a precompiled one where that
+ * does not compile, BCHDEC_NMS_KERNEL=generic selects it, or the rows exceed shared memory. */
 bch_status bch_nms_backward(const bch_code *code, const bch_nms_params *params,
                             const uint16_t *autos, const float *ckpt, int ld, int n_frames,
                             const float *grad_out, float *grad_llr, float *grad_alpha,

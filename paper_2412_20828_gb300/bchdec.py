@@ -27,7 +27,8 @@ FLAG_CONVERGED, FLAG_OSD = 1, 2
 
 # Every symbol the header declares (checked by the tests without a GPU).
 EXPORTS = (
-    "bch_build_pcm", "bch_build_pcm_host", "bch_search_pcm", "bch_nms_kernel_info", "bch_nms_jit_check", "bch_code_info", "bch_pcm_export", "bch_code_free",
+    "bch_build_pcm", "bch_build_pcm_host", "bch_search_pcm", "bch_nms_kernel_info",
+    "bch_nms_kernel_name", "bch_nms_jit_check", "bch_code_info", "bch_pcm_export", "bch_code_free",
     "bch_draw_automorphisms", "bch_draw_automorphisms_host", "bch_gen_frames",
     "bch_workspace_size", "bch_nms_decode", "bch_hybrid_decode", "bch_hybrid_decode_noalloc",
     "bch_osd_decode",
@@ -116,6 +117,7 @@ def load():
             "bch_search_pcm": (st, [i, i, i, u64, C.POINTER(PcmOpts), i, P, P, sz, C.POINTER(i),
                                     C.POINTER(P)]),
             "bch_nms_kernel_info": (st, [P, i, i, C.c_char_p, sz]),
+            "bch_nms_kernel_name": (st, [P, C.POINTER(NmsParams), i, C.c_char_p, sz]),
             "bch_nms_jit_check": (st, [i, i, i, u64, P, i, C.c_char_p, sz]),
             "bch_code_info": (st, [P, C.POINTER(i), C.POINTER(i), C.POINTER(i), C.POINTER(i),
                                    C.POINTER(i)]),
@@ -237,6 +239,12 @@ class Code:
     def kernel_info(self, msg=MSG_FP32, n_autos=3) -> str:
         buf = C.create_string_buffer(4096)
         _check(load().bch_nms_kernel_info(self._h, msg, n_autos, buf, 4096), "bch_nms_kernel_info")
+        return buf.value.decode()
+
+    def kernel_name(self, p: "NmsParams", n_frames: int) -> str:
+        """Names of the min-sum kernels a decode of ``n_frames`` frames with ``p`` runs (loads them)."""
+        buf = C.create_string_buffer(256)
+        _check(load().bch_nms_kernel_name(self._h, C.byref(p), n_frames, buf, 256), "bch_nms_kernel_name")
         return buf.value.decode()
 
     def dense(self) -> np.ndarray:

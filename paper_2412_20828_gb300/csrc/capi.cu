@@ -553,23 +553,6 @@ bch_status bch_build_pcm(int n, int k, bch_pcm_kind kind, int m_rows, uint64_t s
   return BCH_OK;
 }
 
-bch_status bch_nms_kernel_info(const bch_code *code, int msg, int n_autos, char *buf, size_t capacity) {
-  if (!code_ok(code) || !buf || capacity == 0) return fail(BCH_EINVAL, "bad argument");
-  std::string info;
-  const int mode = kernel_mode();
-  if (n_autos == 0) {
-    info = "generic: plain decoder";
-  } else if (mode == 1) {
-    info = "generic: selected by BCHDEC_NMS_KERNEL";
-  } else {
-    std::string err;
-    cudaKernel_t k = jit_kernel(code, msg, &err);
-    info = k ? "jit" : "generic: " + err;
-  }
-  std::snprintf(buf, capacity, "%s", info.c_str());
-  return BCH_OK;
-}
-
 bch_status bch_nms_jit_check(int n, int k, int m_rows, uint64_t seed, const bch_pcm_opts *opts, int msg,
                              char *log, size_t capacity) {
   if (!log || capacity == 0 || msg < BCH_MSG_FP32 || msg > BCH_MSG_INT8) return fail(BCH_EINVAL, "bad argument");
@@ -857,61 +840,79 @@ static cudaError_t launch_rcp(cudaKernel_t k, int FB, const bch_code *code, cons
   return cudaLaunchKernel(fn, dim3(unsigned(blocks)), dim3(unsigned(tpb)), args, smem, st);
 }
 
+// The kernels one call runs, compiled and loaded (nothing is launched).
+struct NmsPlan {
+  enum Kind { kPrecompiled, kRowColumn, kPlain, kStraight } kind = kPrecompiled;
+  cudaKernel_t kernel = nullptr;  // null: precompiled
+  int slots = 0;                  // frame slots per block (row/column kernels)
+  cudaKernel_t rest = nullptr;    // the kernel of the frames a straight-line one defers
+  int rest_slots = 0;
+  std::string why;  // why a run-time kernel did not load; empty if the precompiled one is the choice
+  const char *name(int P) const {
+    switch (kind) {
+      case kRowColumn: return "bch_nms_rc";
+      case kPlain: return "bch_plain_rc";
+      case kStraight: return rest ? "bch_nms_jit + bch_nms_rc" : "bch_nms_jit";
+      default: return P == 0 ? "nms_plain_kernel" : "nms_enhanced_kernel";
+    }
+  }
+};
+
+// Every rule that picks a min-sum kernel: the mode, the row/column lines, then (auto and jit)
+// the straight-line kernel.  A kernel that does not compile leaves the call to the next one.
+static cudaError_t plan_nms(const bch_code *code, const NmsArgs &a, NmsPlan *p) {
+  if (kernel_mode() == 1) {
+    p->why = "selected by BCHDEC_NMS_KERNEL";
+    return cudaSuccess;
+  }
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  if (a.P == 0) {
+    p->slots = rcp_slots(code, a, sms);
+    if (p->slots && (p->kernel = jit_rcp_kernel(code, p->slots, &p->why))) p->kind = NmsPlan::kPlain;
+    return cudaSuccess;
+  }
+  p->slots = rc_slots(code, a, sms);
+  if (p->slots && (p->kernel = jit_rc_kernel(code, a.msg, a.qfrac, p->slots, a.P, &p->why))) {
+    p->kind = NmsPlan::kRowColumn;
+    return cudaSuccess;
+  }
+  // the FP32 kernel of n <= 63 leaves frames with a NaN to the row/column kernel, launched over
+  // its list (empty in all but odd calls: 2 us).  With 32 slots where they fit: 10^6 frames of
+  // BCH(63,36) with a NaN in each 22 ms, with one slot 42 ms.  A call of little work keeps the
+  // edge order and spares the second launch, 3 to 7 us: one iteration of 60 800 frames of
+  // BCH(63,36), one copy, 42.8 / 49.6 us, three copies 74.8 / 78.3 us
+  p->rest_slots = rc_fits(code, a, 32) ? 32 : 1;
+  const long long work = (long long)a.F * a.I * code->dc.edges * a.P;
+  if (work >= 2000000LL * sms && jit_defers(code->alg.n, a.msg) && rc_fits(code, a, p->rest_slots))
+    p->rest = jit_rc_kernel(code, a.msg, a.qfrac, p->rest_slots, a.P, &p->why);
+  if ((p->kernel = jit_kernel(code, a.msg, &p->why, a.qfrac, p->rest != nullptr))) p->kind = NmsPlan::kStraight;
+  return cudaSuccess;
+}
+
 // Launches the min-sum kernel for this call; *cleared: whether the queue counters were zeroed.
 static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaStream_t st,
                                    std::string *why, bool *cleared) {
-  const int mode = kernel_mode();
-  if (a.P == 0 && mode != 1) {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int fb = rcp_slots(code, a, sms);
-    std::string err;
-    if (fb)
-      if (cudaKernel_t k = jit_rcp_kernel(code, fb, &err)) return launch_rcp(k, fb, code, a, st, cleared);
+  NmsPlan p;
+  cudaError_t e = plan_nms(code, a, &p);
+  if (e != cudaSuccess) return e;
+  if (p.kind == NmsPlan::kPlain) return launch_rcp(p.kernel, p.slots, code, a, st, cleared);
+  if (p.kind == NmsPlan::kRowColumn) return launch_rc(p.kernel, p.slots, code, a, st, cleared);
+  e = clear_queue(a, st, cleared);
+  if (e != cudaSuccess) return e;
+  if (p.kind == NmsPlan::kStraight) {
+    e = launch_jit(p.kernel, code, a, st);
+    if (e != cudaSuccess || !p.rest) return e;
+    NmsArgs d = a;
+    d.list = a.defer;
+    d.list_count = a.defer_count;
+    d.queue = a.queue + 3;
+    return launch_rc(p.rest, p.rest_slots, code, d, st, cleared);
   }
-  int sms = 0;
-  if (a.P > 0 && mode != 1) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int fb = rc_slots(code, a, sms);
-    std::string err;
-    if (fb)
-      if (cudaKernel_t k = jit_rc_kernel(code, a.msg, a.qfrac, fb, a.P, &err)) return launch_rc(k, fb, code, a, st, cleared);
-  }
-  const cudaError_t ec = clear_queue(a, st, cleared);
-  if (ec != cudaSuccess) return ec;
-  // auto and jit: the specialised kernel (for n = 127 it spills but still runs 1.8x
-  // faster than the precompiled one; its first compile takes tens of seconds and is
-  // cached on disk); auto falls back to the precompiled kernel if it does not compile
-  if (a.P > 0 && mode != 1) {
-    std::string err;
-    // the FP32 kernel of n <= 63 leaves frames with a NaN to the row/column kernel, launched
-    // over its list (empty in all but odd calls: 2 us).  With 32 slots where they fit: 10^6
-    // frames of BCH(63,36) with a NaN in each 22 ms, with one slot 42 ms
-    cudaKernel_t rk = nullptr;
-    const int rfb = rc_fits(code, a, 32) ? 32 : 1;
-    // (a call of little work keeps the edge order and spares the second launch, 3 to 7 us: one
-    // iteration of 60 800 frames of BCH(63,36), one copy, 42.8 / 49.6 us, three copies 74.8 / 78.3 us)
-    const long long work = (long long)a.F * a.I * code->dc.edges * a.P;
-    if (work >= 2000000LL * sms && jit_defers(code->alg.n, a.msg) && rc_fits(code, a, rfb))
-      rk = jit_rc_kernel(code, a.msg, a.qfrac, rfb, a.P, &err);
-    cudaKernel_t k = jit_kernel(code, a.msg, &err, a.qfrac, rk != nullptr);
-    if (k) {
-      cudaError_t e = launch_jit(k, code, a, st);
-      if (e != cudaSuccess || !rk) return e;
-      NmsArgs d = a;
-      d.list = a.defer;
-      d.list_count = a.defer_count;
-      d.queue = a.queue + 3;
-      return launch_rc(rk, rfb, code, d, st, cleared);
-    }
-    if (why) *why = err;
-    if (mode == 2) return cudaErrorNotSupported;
-  }
+  if (why) *why = p.why;
+  if (a.P > 0 && kernel_mode() == 2) return cudaErrorNotSupported;
   return launch_nms(a, st);
 }
 
@@ -940,6 +941,43 @@ static cudaError_t launch_backward_code(const bch_code *code, const BwdArgs &a, 
     }
   }
   return launch_backward(a, grad_alpha, st);
+}
+
+bch_status bch_nms_kernel_name(const bch_code *code, const bch_nms_params *params, int n_frames, char *buf,
+                               size_t capacity) {
+  bch_status s = check_params(code, params);
+  if (s != BCH_OK) return s;
+  if (n_frames < 1 || !buf || capacity == 0) return fail(BCH_EINVAL, "bad argument");
+  const NmsArgs a = make_nms_args(code, params, nullptr, code->alg.n, n_frames, nullptr, nullptr, nullptr, nullptr,
+                                  nullptr, nullptr);
+  NmsPlan p;
+  BCH_CUDA(plan_nms(code, a, &p), "kernel choice");
+  std::snprintf(buf, capacity, "%s", p.name(a.P));
+  return BCH_OK;
+}
+
+bch_status bch_nms_kernel_info(const bch_code *code, int msg, int n_autos, char *buf, size_t capacity) {
+  if (!code_ok(code) || !buf || capacity == 0) return fail(BCH_EINVAL, "bad argument");
+  // a call of every size class, the other parameters at their usual values
+  bool some = false;
+  std::string generic;
+  for (int shift = 0; shift < 31; shift++) {
+    NmsArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.F = 1 << shift;
+    a.P = std::max(0, n_autos);
+    a.msg = msg;
+    a.I = 12;
+    a.early_stop = 1;
+    NmsPlan p;
+    BCH_CUDA(plan_nms(code, a, &p), "kernel choice");
+    if (p.kernel) some = true;
+    else if (generic.empty()) generic = p.why;
+  }
+  std::string info = some ? "jit" : "generic: " + generic;
+  if (some && !generic.empty()) info += "; some sizes generic: " + generic;
+  std::snprintf(buf, capacity, "%s", info.c_str());
+  return BCH_OK;
 }
 
 static bch_status run_nms(const bch_code *code, const bch_nms_params *params, const float *llr, int ld,

@@ -43,7 +43,7 @@ def main(argv=None):
         else:
             B.nms_decode(code, p, llr, aut, hard, it, fl, ws=ws)
     torch.cuda.synchronize()
-    print(f"BCH({n},{k}) {F} frames at {a.ebn0} dB, {a.msg}: kernel {code.kernel_info(msg)}, "
+    print(f"BCH({n},{k}) {F} frames at {a.ebn0} dB, {a.msg}: kernel {code.kernel_name(p, F)}, "
           f"mean iterations {float(it.float().mean()):.3f}, edges {code.edges}")
 
 
