@@ -40,7 +40,8 @@ def _batch(code, F, ld, seed):
         elif what == 4:
             r[at] = np.nan
         elif what == 5:  # passes 2^100 and the range after a merge: infinities, then NaN
-            r *= np.float32(1e37)
+            with np.errstate(over="ignore"):
+                r *= np.float32(1e37)
         elif what == 6:
             r[:] = np.where(r < 0, -FMAX, FMAX)
         else:
