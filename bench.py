@@ -11,7 +11,9 @@ One step = for each code: draw the automorphisms, enhanced NMS over all points, 
 failed-frame compaction, order-2 OSD on the failed frames (standard H) and per-point
 error counters -- every step of the decoding path.  `value` is frames/s over the whole
 job; `e2e` is the same metric through the host-memory pipeline (bch_decoder) with the
-copies inside the timed region.  `--impl reference` times the FP64 CPU oracle.
+copies inside the timed region.  `--impl reference` times the FP64 CPU oracle.  The result
+is one line on stdout; the tables by Eb/N0 point and the legs' details go to stderr
+("# tables {...}").
 """
 from __future__ import annotations
 
@@ -454,6 +456,36 @@ def run_training(B, torch, steps, batch=65536, iters=12):
             "alpha": [round(float(a), 4) for a in alpha]}
 
 
+def headline(line):
+    """The result line's short form and the tables left out of it.  The line keeps every key of
+    the whole-job result (value, e2e, roofline, clocks, ...) and one row per leg; the points'
+    tables and the legs' details (15 KB of a 20 KB line) go to the second dict."""
+    def pick(d, *keys):
+        return d if d is None or "error" in d else {k: d[k] for k in keys if k in d}
+
+    short, tables = dict(line), {}
+    for key in ("msg_legs", "config4", "pcm_search", "serving", "training", "plain_nms", "per_point"):
+        tables[key] = short.pop(key, None)
+    roof = ("kernel", "frac", "nms_ms_per_step")
+    short["msg_legs"] = {k: {**pick(v, "frames_per_s", "ms_per_step"), **pick(v["roofline"], *roof)}
+                         for k, v in (tables["msg_legs"] or {}).items()}
+    if tables["config4"]:
+        c4 = tables["config4"]
+        short["config4"] = {**pick(c4, "frames_per_step", "frames_per_s", "ms_per_step"),
+                            "codes": {k: pick(v["roofline"], *roof) for k, v in c4["codes"].items()}}
+    short["pcm_search"] = pick(tables["pcm_search"], "chains", "search_s", "four_cycles")
+    if tables["serving"]:
+        sv, served = tables["serving"], ("p50_ms", "p99_ms", "served_frames_per_s")
+        short["serving"] = sv if "error" in sv else {
+            "seconds": sv["seconds"],
+            **{k: pick(sv[k], *served) for k in ("server", "static_batching")},
+            **{k: {"rate_rps": sv[k]["rate_rps"], **{m: pick(sv[k][m], *served) for m in ("server", "static_batching")}}
+               for k in ("below_saturation", "twice_the_rate")}}
+    short["training"] = pick(tables["training"], "steps", "ms_per_step", "frames_per_s", "loss_first", "loss_last")
+    short["plain_nms"] = pick(tables["plain_nms"], "frames_per_s", "us_per_decode", "fer")
+    return short, tables
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -822,6 +854,8 @@ def main():
             "serving": serving, "training": training, "plain_nms": plain,
             "fer_match_oracle_ci95": fer_match, "fer_match_detail": fer_detail, "per_point": per_point,
         }
+        line, tables = headline(line)
+        print("# tables " + json.dumps(tables), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if dist:
         dist.destroy_process_group()
