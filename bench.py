@@ -38,15 +38,14 @@ P_AUTOS, ITERS, ALPHA, OSD_ORDER = 3, 12, 0.78, 2
 SEED_FRAMES, SEED_AUTOS = 20241230, 0x5EED
 METRIC = "frames/s & edge-updates/s on 1 GB300 at oracle-matched FER; served p50/p99 latency"
 LANE_OPS_PER_EDGE = 8  # min1/min2 (3), sign (1), output select (2), accumulate (1), gather (1)
-# DRAM bytes per decoded frame of the specialised NMS kernel, from one ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum) of a 1.1 M-frame BCH(63,36) launch:
-# 288.41 MB + 9.63 MB.  Traffic grows with the frames a launch decodes (each frame's
-# LLRs are read once, its results written once), so a launch's traffic is this figure
-# times its frames.  Set to None when the kernel changes until it is re-captured.
-JIT_DRAM_BYTES_PER_FRAME = (288.41e6 + 9.63e6) / 1.1e6
-# The same for the n = 127 specialised kernel (split mapping), from one ncu capture of
-# a 400 000-frame BCH(127,64) launch at 3 dB: 209.26 MB + 8.15 MB.
-JIT127_DRAM_BYTES_PER_FRAME = (209.26e6 + 8.15e6) / 4e5
+# DRAM bytes per decoded frame of the NMS kernels, by kernel and block length, from one ncu
+# capture each (dram__bytes_read.sum + dram__bytes_write.sum): bch_nms_jit on 1.1 M frames of
+# BCH(63,36) at 3 dB, bch_nms_rc on 400 000 frames of BCH(127,64) at 3 dB.  Traffic grows with the
+# frames a launch decodes (each frame's LLRs are read once, its results written once), so a
+# launch's traffic is this figure times its frames.  Drop an entry when its kernel changes until
+# it is captured again.
+DRAM_BYTES_PER_FRAME = {("bch_nms_jit", 63): (289.52e6 + 9.41e6) / 1.1e6,
+                        ("bch_nms_rc", 127): (207.64e6 + 7.03e6) / 4e5}
 CONFIG4_CODES = [(127, 64), (127, 99)]
 CONFIG4_POINTS = [2.0 + 0.5 * i for i in range(7)]
 
@@ -294,7 +293,7 @@ def run_plain(B, torch, dev, reps=50):
             "edge_updates_per_s": float(c[5]) * 486 / dt}
 
 
-def nms_roofline(torch, dev, clocks, edge_updates, nms_time, kernel, frames, n, traffic_per_frame):
+def nms_roofline(torch, dev, clocks, edge_updates, nms_time, kernel, frames, n, fp32=True):
     """Roofline of the enhanced-NMS kernel: ALU lane-ops (8 per edge update) per second
     against SMs x 128 lanes x the median SM clock under load."""
     peaks = measured_peaks()
@@ -303,8 +302,9 @@ def nms_roofline(torch, dev, clocks, edge_updates, nms_time, kernel, frames, n, 
     peak_lane_ops = sms * 128 * clk_mhz * 1e6
     achieved = edge_updates * LANE_OPS_PER_EDGE / nms_time
     traffic = None
-    if kernel.startswith("bch_") and traffic_per_frame is not None:
-        traffic = traffic_per_frame * frames  # bytes per launch (one code's frames)
+    per_frame = DRAM_BYTES_PER_FRAME.get((kernel.split(" + ")[0], n)) if fp32 else None
+    if per_frame is not None:
+        traffic = per_frame * frames  # bytes per launch (one code's frames)
     W64 = (n + 63) // 64
     ld = 64 if n <= 63 else 128
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_lane_ops / 1e12,
@@ -393,8 +393,7 @@ def run_config4(B, torch, dev, clocks, frames_per_point, steps=2, warmup=1):
                         "ber": c[2] / (c[0] * st["n"]), "nms_fer": 1 - c[6] / c[0],
                         "avg_iters": c[5] / c[0], "osd_frames": int(c[4])})
         out["codes"][f"({st['n']},{st['k']})"] = {
-            "roofline": nms_roofline(torch, dev, clocks, eu, nms_t, kernel, F, st["n"],
-                                     JIT127_DRAM_BYTES_PER_FRAME if st["n"] == 127 else None),
+            "roofline": nms_roofline(torch, dev, clocks, eu, nms_t, kernel, F, st["n"]),
             "per_point": pts}
         st["code"].close()
         st["std"].close()
@@ -644,7 +643,7 @@ def main():
     eups = edge_updates / nms_time
     kernel = states[0]["code"].kernel_name(states[0]["p"], F)
     roofline = nms_roofline(torch, dev, clocks, edge_updates, nms_time, kernel, F, 63,
-                            JIT_DRAM_BYTES_PER_FRAME if msg == B.MSG_FP32 else None)
+                            fp32=msg == B.MSG_FP32)
 
     # the step's decisions on the oracle's sample (frames 0..N-1 of every point), taken
     # now: the legs below decode other message formats into the same buffers
@@ -680,7 +679,7 @@ def main():
         fe = [int((st["hard"] != st["cw"]).any(dim=1).sum()) for st in states]
         msg_legs[name] = {"frames_per_s": frames_per_step / t_leg, "ms_per_step": t_leg * 1e3,
                           "roofline": nms_roofline(torch, dev, clocks, eu, nt,
-                                                   states[0]["code"].kernel_name(states[0]["p"], F), F, 63, None),
+                                                   states[0]["code"].kernel_name(states[0]["p"], F), F, 63, fp32=False),
                           "frame_errors_per_code": fe}
         for st, p0 in zip(states, saved):
             st["p"] = p0

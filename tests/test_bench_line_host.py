@@ -61,3 +61,19 @@ def test_legs_that_were_skipped_or_failed():
     short, _ = bench.headline({**_line(), "config4": None, "pcm_search": None, "serving": {"error": "closed"},
                                "training": None, "plain_nms": None, "msg_legs": {}})
     assert short["serving"] == {"error": "closed"} and short["training"] is None and short["msg_legs"] == {}
+
+
+def test_traffic_belongs_to_the_kernel_that_ran(monkeypatch):
+    """A launch's DRAM traffic is scaled from a capture of the same kernel, block length and
+    format, and left out where there is none."""
+    import types
+    props = types.SimpleNamespace(multi_processor_count=152)
+    torch = types.SimpleNamespace(cuda=types.SimpleNamespace(get_device_properties=lambda dev: props))
+
+    def traffic(kernel, n, fp32=True):
+        return bench.nms_roofline(torch, 0, {"sm_mhz": 2070.0}, 1e9, 1e-3, kernel, 1000, n, fp32=fp32)["traffic"]
+
+    assert traffic("bch_nms_jit + bch_nms_rc", 63) == 1000 * bench.DRAM_BYTES_PER_FRAME["bch_nms_jit", 63]
+    assert traffic("bch_nms_rc", 127) == 1000 * bench.DRAM_BYTES_PER_FRAME["bch_nms_rc", 127]
+    assert traffic("bch_nms_rc", 63) is None and traffic("bch_nms_jit", 127) is None
+    assert traffic("bch_nms_jit", 63, fp32=False) is None and traffic("nms_enhanced_kernel", 63) is None
