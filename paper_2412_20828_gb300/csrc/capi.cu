@@ -723,10 +723,11 @@ static bool rc_fits(const bch_code *code, const NmsArgs &a, int FB) {
 //  * n <= 63, three copies, 32 slots (64 frames of an SM at a time): with 8 iterations or more and
 //    early stop up to 136 per SM, FP16 224, INT8 152 (BCH(63,36) at 1 to 2 dB: FP32 136 per SM - / 322 /
 //    353, 144 per SM - / 341 / 328; FP16 224 per SM - / 571 / 625; INT8 152 per SM - / 543 / 634).  Without
-//    early stop, or with few iterations, where refilling the slots shows, up to 96, FP16 160,
-//    INT8 128 (FP32 BCH(63,36) 96 per SM, 4 iterations at 1 to 2 dB - / 107 / 129, 128 per SM - / 142 / 129;
-//    BCH(63,57) 128 per SM, no early stop, - / 217 / 194; FP16 BCH(63,45) 160 per SM - / 350 / 384, 192 per SM
-//    - / 410 / 386; INT8 BCH(63,36) 152 per SM - / 650 / 631); n = 15 then up to 64;
+//    early stop up to 128, FP16 160, INT8 128 (FP32 BCH(63,36) 120 per SM - / 303 / 348, 136 per SM - / 380 /
+//    348; FP16 BCH(63,45) 160 per SM - / 350 / 384, 192 per SM - / 410 / 386; INT8 BCH(63,36) 152 per SM - / 650 /
+//    631); FP32 with few iterations, where refilling the slots shows, or few edges up to 96
+//    (BCH(63,36), 4 iterations at 1 to 2 dB, 96 per SM - / 107 / 129, 128 per SM - / 142 / 129; BCH(63,57) 128 per
+//    SM, no early stop, - / 217 / 194); n = 15 without early stop up to 64;
 //  * other numbers of copies, whose loops are not unrolled, up to 64: BCH(63,36), no early stop, 64
 //    per SM one copy 147 / 117 / 149, nine copies 1518 / 607 / 940;
 //  * n = 63 beyond ~1000 edges the straight-line rows outgrow the instruction cache: BCH(63,36)
@@ -765,7 +766,7 @@ static int rc_slots(const bch_code *code, const NmsArgs &a, int sms) {
   int many = 64;
   if (a.P == 3 && !cached) many = by_format(INT_MAX, INT_MAX, 300);
   else if (a.P == 3 && a.I >= 8 && a.early_stop) many = by_format(136, 224, 152);
-  else if (a.P == 3 && n == 63) many = by_format(96, 160, 128);
+  else if (a.P == 3 && n == 63) many = by_format(a.I >= 8 && code->dc.edges > 500 ? 128 : 96, 160, 128);
   else if (!cached && (a.P == 2 || (a.P == 1 && a.msg != BCH_MSG_FP32))) many = 128;
   return within(many) ? 32 : 0;
 }
