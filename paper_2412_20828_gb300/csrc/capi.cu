@@ -859,6 +859,23 @@ struct NmsPlan {
   }
 };
 
+static cudaError_t device_sms(int *sms) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e == cudaSuccess ? cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) : e;
+}
+
+// Whether a straight-line call defers frames with a NaN.  The FP32 kernel of n = 63 leaves them
+// to the row/column kernel, launched over its list (empty in all but odd calls: 2 us), with 32
+// slots where they fit: 10^6 frames of BCH(63,36) with a NaN in each 22 ms, with one slot 42 ms.
+// A call of little work keeps the edge order and spares the second launch, 3 to 7 us: one
+// iteration of 60 800 frames of BCH(63,36), one copy, 42.8 / 49.6 us, three copies 74.8 / 78.3 us.
+static int rest_slots(const bch_code *code, const NmsArgs &a, int sms) {
+  const long long work = (long long)a.F * a.I * code->dc.edges * a.P;
+  if (work < 2000000LL * sms || !jit_defers(code->alg.n, a.msg)) return 0;
+  return rc_fits(code, a, 32) ? 32 : rc_fits(code, a, 1) ? 1 : 0;
+}
+
 // Every rule that picks a min-sum kernel: the mode, the row/column lines, then (auto and jit)
 // the straight-line kernel.  A kernel that does not compile leaves the call to the next one.
 static cudaError_t plan_nms(const bch_code *code, const NmsArgs &a, NmsPlan *p) {
@@ -866,9 +883,8 @@ static cudaError_t plan_nms(const bch_code *code, const NmsArgs &a, NmsPlan *p) 
     p->why = "selected by BCHDEC_NMS_KERNEL";
     return cudaSuccess;
   }
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0;
+  const cudaError_t e = device_sms(&sms);
   if (e != cudaSuccess) return e;
   if (a.P == 0) {
     p->slots = rcp_slots(code, a, sms);
@@ -880,15 +896,8 @@ static cudaError_t plan_nms(const bch_code *code, const NmsArgs &a, NmsPlan *p) 
     p->kind = NmsPlan::kRowColumn;
     return cudaSuccess;
   }
-  // the FP32 kernel of n <= 63 leaves frames with a NaN to the row/column kernel, launched over
-  // its list (empty in all but odd calls: 2 us).  With 32 slots where they fit: 10^6 frames of
-  // BCH(63,36) with a NaN in each 22 ms, with one slot 42 ms.  A call of little work keeps the
-  // edge order and spares the second launch, 3 to 7 us: one iteration of 60 800 frames of
-  // BCH(63,36), one copy, 42.8 / 49.6 us, three copies 74.8 / 78.3 us
-  p->rest_slots = rc_fits(code, a, 32) ? 32 : 1;
-  const long long work = (long long)a.F * a.I * code->dc.edges * a.P;
-  if (work >= 2000000LL * sms && jit_defers(code->alg.n, a.msg) && rc_fits(code, a, p->rest_slots))
-    p->rest = jit_rc_kernel(code, a.msg, a.qfrac, p->rest_slots, a.P, &p->why);
+  p->rest_slots = rest_slots(code, a, sms);
+  if (p->rest_slots) p->rest = jit_rc_kernel(code, a.msg, a.qfrac, p->rest_slots, a.P, &p->why);
   if ((p->kernel = jit_kernel(code, a.msg, &p->why, a.qfrac, p->rest != nullptr))) p->kind = NmsPlan::kStraight;
   return cudaSuccess;
 }
@@ -960,6 +969,8 @@ bch_status bch_nms_kernel_name(const bch_code *code, const bch_nms_params *param
 bch_status bch_nms_kernel_info(const bch_code *code, int msg, int n_autos, char *buf, size_t capacity) {
   if (!code_ok(code) || !buf || capacity == 0) return fail(BCH_EINVAL, "bad argument");
   // a call of every size class, the other parameters at their usual values
+  int sms = 0, last = -1;
+  BCH_CUDA(device_sms(&sms), "kernel choice");
   bool some = false;
   std::string generic;
   for (int shift = 0; shift < 31; shift++) {
@@ -970,6 +981,9 @@ bch_status bch_nms_kernel_info(const bch_code *code, int msg, int n_autos, char 
     a.msg = msg;
     a.I = 12;
     a.early_stop = 1;
+    const int choice = a.P == 0 ? rcp_slots(code, a, sms) : 64 * rc_slots(code, a, sms) + rest_slots(code, a, sms);
+    if (choice == last) continue;  // the class of the size before
+    last = choice;
     NmsPlan p;
     BCH_CUDA(plan_nms(code, a, &p), "kernel choice");
     if (p.kernel) some = true;
