@@ -1082,7 +1082,8 @@ cudaKernel_t jit_kernel_from_source(const bch_code *c, int msg, std::string *err
 
 // The row/column kernel of code c with FB slots per block for P copies;
 // nullptr with *err when it does not compile.  Three copies, the usual number, get a kernel
-// of their own (the copies' loops unrolled); any other number shares one.
+// of their own (the copies' loops unrolled); any other number shares one.  (No environment knob
+// shapes the sources of this kernel and the two below, so their keys hold none.)
 cudaKernel_t jit_rc_kernel(const bch_code *c, int msg, int qfrac, int FB, int P, std::string *err) {
   const int PC = P == 3 ? 3 : 0;
   const std::string key = "rc/" + std::to_string(msg) + "/" + std::to_string(qfrac) + "/" + std::to_string(FB) +

@@ -16,7 +16,8 @@
 //                matrix into the frame's syndrome (H_o has rank n - k, so both matrices
 //                vanish on the same words)
 // Every warp follows the slots' frames and iteration counts in its lanes, so an iteration
-// has three block barriers and more only when frames finish.  Shared arrays are
+// has three block barriers (four in the reduced formats, which store y after its scale is
+// known) and more only when frames finish.  Shared arrays are
 // [index][slot], so with RC_FB = 32 a warp is 32 frames of one task and every access is
 // free of bank conflicts.  With RC_FB = 1 a block is one frame: a warp spans 32 tasks, the
 // copies of one row or variable next to each other (some bank conflicts, but no frame waits
