@@ -104,3 +104,21 @@ def test_infinite_bits_keep_the_batch_kernel_s_speed(nk):
             best = min(best, a.elapsed_time(b))
         times.append(best)
     assert times[1] <= 3.0 * times[0], times
+
+
+def test_checkpoints_of_deferred_frames(monkeypatch):
+    """The training forward pass on a batch large enough to defer its NaN frames: every
+    checkpoint is the same bits as in edge order."""
+    import torch
+    code, F, iters = B.Code(63, 45), 70_001, 6
+    llr = _batch(code, F, 64, 9)
+    autos = autos_dev(B.draw_automorphisms_host(63, 3, 54, 0, F))
+    p = B.params(iters, 0.7)
+    assert code.kernel_name(B.params(iters, 0.7, early_stop=False), F) == "bch_nms_jit + bch_nms_rc"
+    got = []
+    for grid in ("0", "1"):
+        monkeypatch.setenv("BCHDEC_JIT_GRID", grid)
+        ck = torch.zeros((iters + 1, F, 64), device="cuda")
+        B.nms_forward_train(code, p, llr, autos, ck)
+        got.append(ck.view(torch.int32))
+    assert torch.equal(got[0], got[1])
