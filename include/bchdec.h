@@ -482,7 +482,8 @@ bch_status bch_nms_forward_train(const bch_code *code, const bch_nms_params *par
  * at a = argmin over the row without u (lowest column on ties); sign derivatives 0.
  * Recomputes each iteration from its checkpoint.  Runs a kernel compiled at run time for the
  * code (bch_bwd_rc; on first use, as the decoders' kernels), or a precompiled one where that
- * does not compile, BCHDEC_NMS_KERNEL=generic selects it, or the rows exceed shared memory. */
+ * does not compile, BCHDEC_NMS_KERNEL=generic selects it, the rows exceed shared memory, or
+ * the batch is a large one of n = 15 with at most four automorphisms. */
 bch_status bch_nms_backward(const bch_code *code, const bch_nms_params *params,
                             const uint16_t *autos, const float *ckpt, int ld, int n_frames,
                             const float *grad_out, float *grad_llr, float *grad_alpha,

@@ -930,17 +930,24 @@ static cudaError_t launch_nms_code(const bch_code *code, const NmsArgs &a, cudaS
 // compiler, BCHDEC_NMS_KERNEL=generic, or a matrix whose tables or row states do not fit) the
 // precompiled one-thread-per-frame kernel.  us, P = 3, 12 iterations, new / precompiled:
 // BCH(127,64) 256 frames 304 / 11 234, 65 536 frames 4 138 / 45 017; BCH(63,36) 256 frames 122 /
-// 3 314, 65 536 frames 1 680 / 7 585: no size prefers the precompiled one.
+// 3 314, 65 536 frames 1 680 / 7 585: no size of these prefers the precompiled one.  n = 15 with few
+// copies does beyond 320 frames per SM, where its short rows fill the GPU: BCH(15,7), one copy
+// 30 000 frames 105 / 145, 65 536 frames 209 / 183; three copies 65 536 frames 447 / 483, 6.4 / 3.5 us per
+// 1000 more; nine copies 1165 / 1765, 17 / 21.
 static cudaError_t launch_backward_code(const bch_code *code, const BwdArgs &a, float *grad_alpha, cudaStream_t st) {
   const int n = code->alg.n, R = int(code->rows.size());
   const size_t smem = size_t(rcb_words(n, a.P, R, code->rc.w4, kRcbWarps, kRcbAcc)) * 4;
-  if (a.F > 0 && kernel_mode() != 1 && smem <= 227 * 1024 && code->rc.const_bytes <= kRcConstBytes) {
+  int sms = 0;
+  cudaError_t e = device_sms(&sms);
+  if (e != cudaSuccess) return e;
+  const bool many_short = n < 63 && a.P <= 4 && a.F > 320LL * sms;
+  if (a.F > 0 && !many_short && kernel_mode() != 1 && smem <= 227 * 1024 && code->rc.const_bytes <= kRcConstBytes) {
     std::string err;
     cudaKernel_t k = jit_rcb_kernel(code, &err);
     if (k) {
       const void *fn = reinterpret_cast<const void *>(k);
-      int sms = 0, per_sm = 0;
-      cudaError_t e = launch_geometry(fn, 32 * kRcbWarps, smem, &sms, &per_sm);
+      int per_sm = 0;
+      e = launch_geometry(fn, 32 * kRcbWarps, smem, &sms, &per_sm);
       if (e != cudaSuccess) return e;
       if (per_sm < 1) return cudaErrorInvalidConfiguration;
       const int nb = std::min((a.F + 31) / 32, sms * per_sm);

@@ -63,3 +63,22 @@ def test_plain_decoder_of_the_shortest_code_not_slower_than_precompiled(monkeypa
         monkeypatch.setenv("BCHDEC_NMS_KERNEL", mode)
         t.append(_time(lambda: B.nms_decode(code, p, llr, None, hard, ws=ws)))
     assert t[0] <= 1.15 * t[1], t
+
+
+@pytest.mark.parametrize("P", [1, 3])
+def test_backward_of_the_shortest_code_not_slower_than_precompiled(P, monkeypatch):
+    import torch
+    code, iters = B.Code(15, 7), 12
+    llr, _ = _inputs(code, 2000, 5.0)
+    F, ld = llr.shape
+    autos = autos_dev(B.draw_automorphisms_host(15, P, 83, 0, F))
+    p = B.params(iters, 0.7, n_autos=P)
+    ckpt = torch.zeros((iters + 1, F, ld), device="cuda")
+    B.nms_forward_train(code, p, llr, autos, ckpt)
+    go, gl, ga = torch.ones_like(llr), torch.zeros_like(llr), torch.zeros(iters, device="cuda")
+    ws = B.workspace(code, p, F)
+    t = []
+    for mode in ("auto", "generic"):
+        monkeypatch.setenv("BCHDEC_NMS_KERNEL", mode)
+        t.append(_time(lambda: B.nms_backward(code, p, autos, ckpt, go, gl, ga, ws)))
+    assert t[0] <= 1.15 * t[1], t
