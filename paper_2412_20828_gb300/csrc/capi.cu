@@ -711,9 +711,9 @@ static bool rc_fits(const bch_code *code, const NmsArgs &a, int FB) {
 // The row/column kernel (frame slots per block: 1 or 32) for this call, or 0 when the
 // one-thread-per-frame kernel is the better one.  BCHDEC_JIT_RC=0|1|32 overrides (a tuning
 // and comparison knob; all compute the same bits).  The lines, in frames per SM, lie where no
-// call is slower than on the one-thread-per-frame kernel, also when every frame runs all its
-// iterations (no early stop, or 1 to 2 dB).  Easy frames gain past a line too, but the host
-// cannot know them.  us on a GB300 for 1 slot / 32 slots / one thread per frame, 12 iterations
+// call measured more than 4% or 3 us slower than on the one-thread-per-frame kernel, also when
+// every frame runs all its iterations (no early stop, or 1 to 2 dB).  Easy frames gain past a
+// line too, but the host cannot know them.  us on a GB300 for 1 slot / 32 slots / one thread per frame, 12 iterations
 // unless said; ep = edges x copies:
 //  * one slot: a frame's iteration costs an SM 0.21 us per 1000 ep, at least 0.18 us.  Up to 8 +
 //    61200 / ep frames, where 32 slots win at 1 to 6 dB (BCH(63,36) 4096 frames 77 / 91 / 349, 16 384
@@ -727,7 +727,7 @@ static bool rc_fits(const bch_code *code, const NmsArgs &a, int FB) {
 //    348; FP16 BCH(63,45) 160 per SM - / 350 / 384, 192 per SM - / 410 / 386; INT8 BCH(63,36) 152 per SM - / 650 /
 //    631); FP32 with few iterations, where refilling the slots shows, or few edges up to 96
 //    (BCH(63,36), 4 iterations at 1 to 2 dB, 96 per SM - / 107 / 129, 128 per SM - / 142 / 129; BCH(63,57) 128 per
-//    SM, no early stop, - / 217 / 194); n = 15 without early stop up to 64;
+//    SM, no early stop, - / 217 / 194); n = 15 in both cases up to 64;
 //  * other numbers of copies, whose loops are not unrolled, up to 64: BCH(63,36), no early stop, 64
 //    per SM one copy 147 / 117 / 149, nine copies 1518 / 607 / 940;
 //  * n = 63 beyond ~1000 edges the straight-line rows outgrow the instruction cache: BCH(63,36)
